@@ -46,6 +46,7 @@ struct BatchArgs {
     const upslam_keyframe *kfs;  // device array [n_kf]
     int n_kf, n_hyp, n_prob;
     upslam_pano sp;
+    BinRule srule;  // binning into the sweep
     const float4 *spix;
     const void *snrm;
     int sprec;
@@ -87,9 +88,8 @@ __device__ __forceinline__ BatchHit batch_gather(const BatchArgs &a, const float
     n = make_float3(ent[3 * cap + q], ent[4 * cap + q], ent[5 * cap + q]);
     const float3 qq = xform_inv(Tp, s.x, s.y, s.z);
     int jv = 0, ju = 0;
-    float rr;
     BatchHit h;
-    h.binned = bin_point(qq.x, qq.y, qq.z, a.sp, jv, ju, rr);
+    h.binned = bin_pixel(qq.x, qq.y, qq.z, a.srule, jv, ju);
     const int j = h.binned ? jv * a.sp.cols + ju : 0;
     h.P = __ldg(a.spix + j);
     h.m = load_nw(a.snrm, j, a.sprec);
@@ -583,6 +583,7 @@ extern "C" upslam_status upslam_icp_batched(const upslam_keyframe *d_kfs, const 
     a.n_hyp = n_hyp;
     a.n_prob = n_prob;
     a.sp = sw->pano;
+    a.srule = make_bin_rule(sw->pano);
     a.spix = reinterpret_cast<const float4 *>(sw->d_pix);
     a.snrm = sw->d_nrm;
     a.sprec = sw->nrm_precision;

@@ -9,6 +9,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <float.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <atomic>
@@ -67,6 +69,79 @@ __device__ __forceinline__ bool bin_point(float x, float y, float z, const upsla
     if (col >= pp.cols) col -= pp.cols;
     if (col < 0) col += pp.cols;
     return true;
+}
+
+// A panorama's binning rule with what the fast form below needs, made on the host (make_bin_rule).
+struct BinRule {
+    upslam_pano pp;
+    float r2_min, r2_max;  // sqrt_rn(r2) lies in [r_min, r_max] exactly when r2 lies in [r2_min, r2_max]
+    float az0, el0;        // pi s_az - 1/2 and el_top s_el - 1/2, in pixels
+    float az_half, az_pi;  // pi/2 s_az and pi s_az
+    float lim;             // 1/2 minus the guard; negative: the fast form is off
+};
+
+__device__ __forceinline__ float rcp_approx(float x) {  // relative error below 2^-23
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {  // relative error below 2^-22.9
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The polynomial of atan2p, fused: P(s) with atan(t) = t P(t^2), |t| <= 1.
+__device__ __forceinline__ float atan_poly(float s) {
+    float p = fmaf(0.0028662257f, s, -0.0161657367f);
+    p = fmaf(p, s, 0.0429096138f);
+    p = fmaf(p, s, -0.0752896400f);
+    p = fmaf(p, s, 0.1065626393f);
+    p = fmaf(p, s, -0.1420889944f);
+    p = fmaf(p, s, 0.1999355085f);
+    p = fmaf(p, s, -0.3333314528f);
+    return fmaf(p, s, 1.0f);
+}
+
+// The pixel of an FP32 point, the same as bin_point's bit for bit, usually without its roundings: the two
+// angles are formed with approximate reciprocals and fused multiply-adds, in pixels, and the point's cell is
+// the rule's whenever both coordinates keep `guard` away from a cell's edge, `guard` being more than the two
+// forms can differ by (make_bin_rule derives it; about 4e-4 of a pixel at 1024 columns, so one point in a
+// thousand or so is binned again by the rule itself).  The range test needs no root: it compares the rounded
+// squared range with the squares' exact limits.  A point more than 45 degrees up or down, and whatever makes a
+// NaN here (a point on the axis), goes to the rule.  The rule spends two divisions, two square roots and
+// thirty-two unfused polynomial operations, about 200 instructions; this form about 55.  It bounds
+// every kernel that bins (the registration's steps, the grid search, the batched form).
+__device__ __forceinline__ bool bin_pixel(float x, float y, float z, const BinRule &b, int &row, int &col) {
+    const float xy2 = __fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y));
+    const float z2 = __fmul_rn(z, z);
+    const float r2 = __fadd_rn(xy2, z2);
+    if (!(r2 >= b.r2_min && r2 <= b.r2_max)) return false;
+    const float te = z * rsqrt_approx(xy2);
+    const float fr = fmaf(-(te * b.pp.s_el), atan_poly(te * te), b.el0);
+    const bool swap = fabsf(y) > fabsf(x);
+    const float ta = (swap ? -x : y) * rcp_approx(swap ? y : x);
+    const float k = swap ? b.az_half : (x < 0.0f ? b.az_pi : 0.0f);
+    const float fc = fmaf(-(ta * b.pp.s_az), atan_poly(ta * ta), b.az0 - copysignf(k, y));
+    // nearest integer of f - 1/2 (the cell) and the distance from the cell's middle, both exact
+    constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
+    const float mr = __fadd_rn(fr, kMagic), mc = __fadd_rn(fc, kMagic);
+    const float dr = __fsub_rn(fr, __fsub_rn(mr, kMagic)), dc = __fsub_rn(fc, __fsub_rn(mc, kMagic));
+    row = __float_as_int(mr) - __float_as_int(kMagic);
+    col = __float_as_int(mc) - __float_as_int(kMagic);
+    const bool in_rows = (unsigned)row < (unsigned)b.pp.rows;
+    // (NaN distances fail these tests, so they go to the rule)
+    const bool sure = z2 <= xy2 && fabsf(dr) <= b.lim &&
+                      (!in_rows || (fabsf(dc) <= b.lim && (unsigned)col < (unsigned)b.pp.cols));
+    if (sure) return in_rows;
+    float r;
+    return bin_point(x, y, z, b.pp, row, col, r);
+}
+
+// The same with the point's range (rounded as the rule rounds it).
+__device__ __forceinline__ bool bin_pixel(float x, float y, float z, const BinRule &b, int &row, int &col, float &r) {
+    r = __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y)), __fmul_rn(z, z)));
+    return bin_pixel(x, y, z, b, row, col);
 }
 
 // Pose rounded to FP32, row-major [R | t].
@@ -666,15 +741,15 @@ __device__ __forceinline__ T ld_front(const T *p) {
 }
 
 // Pass 1 of the z-buffer: the point's key (bits(range) << 32 | index) into its pixel.
-__device__ __forceinline__ void project_point(const float4 *pts, int i, const upslam_pano &pp,
+__device__ __forceinline__ void project_point(const float4 *pts, int i, const BinRule &rule,
                                               unsigned long long *zbuf) {
     const float4 p = __ldg(pts + i);
     if (p.w == 0.0f) return;
     int v, u;
     float r;
-    if (!bin_point(p.x, p.y, p.z, pp, v, u, r)) return;
+    if (!bin_pixel(p.x, p.y, p.z, rule, v, u, r)) return;
     const unsigned long long key = ((unsigned long long)__float_as_uint(r) << 32) | (unsigned int)i;
-    atomicMin(zbuf + (size_t)v * pp.cols + u, key);
+    atomicMin(zbuf + (size_t)v * rule.pp.cols + u, key);
 }
 
 // Pass 2: decode the pixel's word into depth / index / point and (kReset) reset the word.
@@ -775,6 +850,7 @@ __device__ __forceinline__ float4 normal_pixel(const Acc &px, const upslam_pano 
 // Everything one keyframe update reads and writes.
 struct FuseView {
     upslam_pano kp;
+    BinRule krule, srule;  // binning into the keyframe (hole fill) and into the sweep (averaging)
     float *kdepth;
     void *knw;
     int kprec;
@@ -794,8 +870,7 @@ __device__ __forceinline__ void fuse_average(const FuseView &f, const PoseF &T, 
     const float w = nk.w;
     const float3 q = xform_inv(T, s.x, s.y, s.z);
     int jv, ju;
-    float rr;
-    if (!bin_point(q.x, q.y, q.z, f.sp, jv, ju, rr)) return;
+    if (!bin_pixel(q.x, q.y, q.z, f.srule, jv, ju)) return;
     const int j = jv * f.sp.cols + ju;
     const float4 P = __ldcg(f.spix + j);
     const float4 m = load_nw_cg(f.snrm, j, f.sprec);
@@ -827,7 +902,7 @@ __device__ __forceinline__ bool holefill_key(const FuseView &f, const PoseF &T, 
     if (m.w == 0.0f) return false;
     const float3 p = xform(T, P.x, P.y, P.z);
     int v, u;
-    if (!bin_point(p.x, p.y, p.z, f.kp, v, u, range)) return false;
+    if (!bin_pixel(p.x, p.y, p.z, f.krule, v, u, range)) return false;
     k = v * f.kp.cols + u;
     key = ((unsigned long long)__float_as_uint(range) << 32) | (unsigned int)j;
     return true;
@@ -890,6 +965,55 @@ static inline bool launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
 static inline bool upslam_pano_ok(const upslam_pano *pp) {
     return pp && pp->rows > 0 && pp->cols > 0 && (int64_t)pp->rows * pp->cols < (int64_t(1) << 31) &&
            pp->s_az > 0.0f && pp->s_el > 0.0f && pp->r_max >= pp->r_min;
+}
+
+// The binning rule of a panorama for bin_pixel.
+//
+// Guard: the largest amount by which the rule's column or row coordinate and bin_pixel's can differ.  With
+// u = 2^-24 (one rounding), on the ratio t = min / max of an octant (|t| <= 1, |d atan / dt| t <= 1/2):
+//   atan, the rule: t one division (3e-8; for the row also a root, 6e-8), the unfused polynomial (1.92 u of its
+//     partial sums: 1.2e-7), its product with t and the square's rounding (6e-8): 2.4e-7 rad;
+//   atan, bin_pixel: t from an approximate reciprocal or reciprocal root (1e-7), the fused polynomial (8e-8),
+//     its products (1.1e-7): 2.9e-7 rad;
+//   column: the rule rounds pi/2 - a, pi - a and pi - az (4.2e-7 rad) and the product with s_az (u fc);
+//     bin_pixel rounds az0, az_half or az_pi, their difference and the sum (4 u of at most 2 pi s_az each);
+//   row: the rule rounds el_top - el and the product with s_el; bin_pixel rounds el0 and the sum: 4 u of at
+//     most (|el_top| + pi/2) s_el.
+// Together below 2.9e-6 rad s_az and (5.3e-7 + 2.4e-7 (|el_top| + 1.6)) rad s_el; both are taken with a fifth
+// more.  A panorama whose coordinates reach 2^20 pixels or whose guard passes a quarter of a pixel, and an
+// unlimited range, take the rule for every point.
+static inline upslam::BinRule make_bin_rule(const upslam_pano &pp) {
+    upslam::BinRule b;
+    b.pp = pp;
+    // (sqrtf rounds to nearest, as the device's root does, and is monotonic: the limits are found by stepping)
+    float lo = 0.0f;
+    if (pp.r_min > 0.0f) {
+        lo = pp.r_min * pp.r_min;
+        if (lo > FLT_MAX) lo = FLT_MAX;
+        while (lo > 0.0f && sqrtf(lo) >= pp.r_min) lo = nextafterf(lo, 0.0f);
+        while (sqrtf(lo) < pp.r_min) lo = nextafterf(lo, INFINITY);
+    }
+    float hi = -1.0f;
+    if (pp.r_max >= 0.0f) {
+        hi = pp.r_max * pp.r_max;
+        if (hi > FLT_MAX && pp.r_max <= FLT_MAX) hi = FLT_MAX;
+        while (hi <= FLT_MAX && sqrtf(hi) <= pp.r_max) hi = nextafterf(hi, INFINITY);
+        while (sqrtf(hi) > pp.r_max) hi = nextafterf(hi, 0.0f);
+    }
+    b.r2_min = lo;
+    b.r2_max = hi;
+    const double s_az = pp.s_az, s_el = pp.s_el, top = pp.el_top;
+    b.az0 = (float)((double)upslam::kPiF * s_az - 0.5);
+    b.el0 = (float)(top * s_el - 0.5);
+    b.az_half = (float)((double)upslam::kHalfPiF * s_az);
+    b.az_pi = (float)((double)upslam::kPiF * s_az);
+    const double g_az = 3.5e-6 * s_az, g_el = (6.4e-7 + 2.9e-7 * (fabs(top) + 1.6)) * s_el;
+    const double g = (g_az > g_el ? g_az : g_el) + 1e-6;
+    const double most = 1048576.0;
+    const bool on = pp.rows < most && pp.cols < most && 6.4 * s_az < most && (fabs(top) + 1.6) * s_el < most &&
+                    g < 0.25 && hi <= FLT_MAX;
+    b.lim = on ? (float)(0.5 - g) : -1.0f;
+    return b;
 }
 
 static inline bool upslam_aligned(const void *p, size_t a) { return ((uintptr_t)p % a) == 0; }

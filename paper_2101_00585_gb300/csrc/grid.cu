@@ -44,6 +44,7 @@ struct GridArgs {
     int kprec;
     const float *kdirs;
     upslam_pano sp;
+    BinRule srule;  // binning into the sweep
     const float4 *spix;
     const void *snrm;
     int sprec;
@@ -128,8 +129,7 @@ __global__ void __launch_bounds__(kGridThreads) grid_score_kernel(GridArgs g, in
                 const float3 s = make_float3(sx[e], sy[e], sz[e]);
                 const float3 q = xform_inv(T, s.x, s.y, s.z);
                 int jv, ju;
-                float rr;
-                if (!bin_point(q.x, q.y, q.z, g.sp, jv, ju, rr)) continue;
+                if (!bin_pixel(q.x, q.y, q.z, g.srule, jv, ju)) continue;
                 const int j = jv * g.sp.cols + ju;
                 const float4 P = __ldg(g.spix + j);
                 const float4 mm = load_nw(g.snrm, j, g.sprec);
@@ -256,6 +256,7 @@ extern "C" upslam_status upslam_grid_score(const upslam_keyframe *kf, const upsl
     g.kprec = kf->precision;
     g.kdirs = kf->d_dirs;
     g.sp = sw->pano;
+    g.srule = make_bin_rule(sw->pano);
     g.spix = reinterpret_cast<const float4 *>(sw->d_pix);
     g.snrm = sw->d_nrm;
     g.sprec = sw->nrm_precision;

@@ -67,6 +67,7 @@ struct IcpArgs {
     int kprec;
     const float *kdirs;
     upslam_pano sp;
+    BinRule srule;  // binning into the sweep
     const float4 *spix;
     const void *snrm;
     int sprec;
@@ -133,8 +134,7 @@ __device__ __forceinline__ void accumulate_pixel(const IcpArgs &a, const PoseF &
     const float3 s = pixel_point(a.kdirs, a.kp.rows, v, u, d);
     const float3 q = xform_inv(T, s.x, s.y, s.z);
     int jv, ju;
-    float rr;
-    if (!bin_point(q.x, q.y, q.z, a.sp, jv, ju, rr)) return;
+    if (!bin_pixel(q.x, q.y, q.z, a.srule, jv, ju)) return;
     const int j = jv * a.sp.cols + ju;
     const float4 P = __ldcg(a.spix + j);
     if (P.w == 0.0f) return;
@@ -356,9 +356,8 @@ struct SweepHit {
 __device__ __forceinline__ SweepHit gather_entry(const IcpArgs &a, const PoseF &T, float3 s) {
     const float3 q = xform_inv(T, s.x, s.y, s.z);
     int jv = 0, ju = 0;
-    float rr;
     SweepHit h;
-    h.binned = bin_point(q.x, q.y, q.z, a.sp, jv, ju, rr);
+    h.binned = bin_pixel(q.x, q.y, q.z, a.srule, jv, ju);
     const int j = h.binned ? jv * a.sp.cols + ju : 0;
     h.P = __ldcg(a.spix + j);
     h.m = load_nw_cg(a.snrm, j, a.sprec);
@@ -693,7 +692,7 @@ __global__ void __launch_bounds__(kTileThreads, 1)
         if (warp > 0) {
             const int pstride = gridDim.x * (kTileThreads - 32);
             for (int i = blockIdx.x * (kTileThreads - 32) + threadIdx.x - 32; i < fr.n; i += pstride)
-                project_point(fr.pts, i, a.sp, fr.zbuf);
+                project_point(fr.pts, i, a.srule, fr.zbuf);
         }
         cta_grid_arrive(ctrl);
         stage_groups(0, my_groups / 2);
@@ -964,6 +963,7 @@ static IcpArgs make_args(const upslam_keyframe *kf, const upslam_sweep *sw, cons
     a.kprec = kf->precision;
     a.kdirs = kf->d_dirs;
     a.sp = sw->pano;
+    a.srule = make_bin_rule(sw->pano);
     a.spix = reinterpret_cast<const float4 *>(sw->d_pix);
     a.snrm = sw->d_nrm;
     a.sprec = sw->nrm_precision;
