@@ -424,17 +424,14 @@ __global__ void __launch_bounds__(512, 1) icp_batched_kernel(BatchArgs a) {
                 const double *tq = totq[warp];
                 double *Tw = Tsh[warp];
                 const long long inliers = (long long)(tq[28] + 0.5);
-                double xi[6] = {0, 0, 0, 0, 0, 0};
+                double xi = 0.0;  // lane k < 6: xi[k]
                 int status = UPSLAM_OK, conv = 0;
-                if (inliers < a.ip.min_inliers) {
+                if (inliers < a.ip.min_inliers || !warp_solve6(tq, a.ip.pivot_eps, &xi)) {
                     status = UPSLAM_ERR_DEGENERATE;
-                } else if (!warp_solve6(tq, a.ip.pivot_eps, xi)) {
-                    status = UPSLAM_ERR_DEGENERATE;
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) xi[i] = 0.0;
+                    xi = 0.0;
                 } else {
-                    warp_se3_update(xi, Tw);
-                    conv = warp_converged(xi, a.ip.eps_rot * a.ip.eps_rot, a.ip.eps_trans * a.ip.eps_trans) ? 1 : 0;
+                    conv = warp_se3_update(xi, Tw, nullptr, a.ip.eps_rot * a.ip.eps_rot,
+                                           a.ip.eps_trans * a.ip.eps_trans) ? 1 : 0;
                 }
                 upslam_icp_stats *st = a.stats + p;
                 if (lane < 12) {
@@ -443,7 +440,7 @@ __global__ void __launch_bounds__(512, 1) icp_batched_kernel(BatchArgs a) {
                 }
                 if (lane < 21) st->A[lane] = tq[lane];
                 else if (lane < 27) st->b[lane - 21] = tq[lane];
-                if (lane < 6) st->xi[lane] = xi[lane];
+                if (lane < 6) st->xi[lane] = xi;
                 if (lane == 0) {
                     st->sse = tq[27];
                     st->inliers = inliers;

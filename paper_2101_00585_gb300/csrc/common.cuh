@@ -71,6 +71,15 @@ __device__ __forceinline__ bool bin_point(float x, float y, float z, const upsla
     return true;
 }
 
+// The rule as a call, for the few points bin_pixel leaves to it: (row << 32) | col, or -1 outside the panorama.
+// Out of line: the kernels bin at many places, and the rule's divisions and roots at each of them made the ICP
+// kernel's instructions a fifth longer.
+static __device__ __noinline__ long long bin_rule_cell(float x, float y, float z, upslam_pano pp) {
+    int row, col;
+    float r;
+    return bin_point(x, y, z, pp, row, col, r) ? ((long long)row << 32) | (unsigned)col : -1ll;
+}
+
 // A panorama's binning rule with what the fast form below needs, made on the host (make_bin_rule).
 struct BinRule {
     upslam_pano pp;
@@ -133,9 +142,11 @@ __device__ __forceinline__ bool bin_pixel(float x, float y, float z, const BinRu
     // (NaN distances fail these tests, so they go to the rule)
     const bool sure = z2 <= xy2 && fabsf(dr) <= b.lim &&
                       (!in_rows || (fabsf(dc) <= b.lim && (unsigned)col < (unsigned)b.pp.cols));
-    if (sure) return in_rows;
-    float r;
-    return bin_point(x, y, z, b.pp, row, col, r);
+    if (__builtin_expect(sure, 1)) return in_rows;
+    const long long cell = bin_rule_cell(x, y, z, b.pp);
+    row = (int)(cell >> 32);
+    col = (int)cell;
+    return cell >= 0;
 }
 
 // The same with the point's range (rounded as the rule rounds it).
@@ -308,6 +319,21 @@ __device__ __forceinline__ double rcp64(double d) {
     const int m = rb & 0x7fffff;
     const double x = __hiloint2double((((rb >> 23) & 0xff) + (1023 - 127)) << 20 | (m >> 3), m << 29);
     return fma(x, fma(-d, x, 1.0), x);
+}
+
+// 1/d for a positive normal d whose reciprocal is normal, as rcp64 without its range: the seed comes from d's
+// mantissa, rounded to FP32 (relative error below 2^-22.4 with the approximate reciprocal, 2^-44 after the step),
+// and d's exponent is taken off the result.
+__device__ __forceinline__ double rcp64_scaled(double d) {
+    const int hi = __double2hiint(d), lo = __double2loint(d);
+    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, lo);  // in [1, 2)
+    const float f = __int_as_float(0x3f800000 + (((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29)) +
+                                   (int)(((unsigned)lo >> 28) & 1u));
+    const int rb = __float_as_int(rcp_approx(f));  // about [1/2, 1]
+    const int rm = rb & 0x7fffff;
+    const double x = __hiloint2double((((rb >> 23) & 0xff) + (1023 - 127)) << 20 | (rm >> 3), rm << 29);
+    const double y = fma(x, fma(-m, x, 1.0), x);
+    return __hiloint2double(__double2hiint(y) - (((hi >> 20) & 0x7ff) - 1023) * (1 << 20), __double2loint(y));
 }
 
 // sin(t)/t, (1 - cos t)/t^2, (t - sin t)/t^3 from t^2: Taylor series (truncation
@@ -489,7 +515,7 @@ __device__ __forceinline__ double dscale2(double x, int e) {
     return __longlong_as_double((b & ~(0x7ffLL << 52)) | ((long long)en << 52));
 }
 
-// FP64 solve of A xi = -b for the symmetric 6x6 A (the square-root-free Cholesky
+// FP64 solve of A xi = -b for the symmetric 6x6 A by elimination (the square-root-free Cholesky
 // factorisation A = L D L^T, i.e. symmetric Gaussian elimination), spread over the
 // lanes of one warp: lanes 0..20 hold the upper triangle of A (lane uidx(i, k)),
 // lanes 21..26 the right-hand side.  GB300 issues an FP64 warp instruction every
@@ -503,10 +529,12 @@ __device__ __forceinline__ double dscale2(double x, int e) {
 // D_j / F_j, and the back substitution, which the common factor of a row does
 // not change, scales every row by its reciprocal pivot in one instruction and
 // then takes one multiply-add per unknown.  Comparisons, maxima and sign flips
-// are integer instructions on the bit patterns.  Every lane returns the same xi.
+// are integer instructions on the bit patterns.
 // False when a standard pivot D_j / F_j <= max(pivot_eps * max diagonal, 1e-300),
 // a pivot is not finite, or the solution is not finite.
-__device__ __forceinline__ bool warp_solve6(const double *tot, double pivot_eps, double xi[6]) {
+// (Out of line: it solves only what warp_solve6 below leaves to it.  Returns xi[k] in lane k < 6 as *x.)
+static __device__ __noinline__ bool warp_solve6_pivots(const double *tot, double pivot_eps, double *x) {
+    double xi[6];
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const bool is_u = lane < 21, is_y = lane >= 21 && lane < 27;
@@ -569,9 +597,99 @@ __device__ __forceinline__ bool warp_solve6(const double *tot, double pivot_eps,
         }
     }
     bool fin = true;
+    double r = xi[0];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) fin = fin && dfinite(xi[i]);
+    for (int i = 0; i < 6; ++i) {
+        fin = fin && dfinite(xi[i]);
+        r = lane == i ? xi[i] : r;
+    }
+    *x = r;
     return fin;
+}
+
+// Field `lane` (5 bits each, lanes 0..11) of a packed table of lane numbers.
+__device__ __forceinline__ int lane_tab(unsigned long long tab, int lane) { return (int)(tab >> (5 * lane)) & 31; }
+constexpr unsigned long long lane_tab6(int a, int b, int c, int d, int e, int f) {
+    return (unsigned long long)a | (unsigned long long)b << 5 | (unsigned long long)c << 10 |
+           (unsigned long long)d << 15 | (unsigned long long)e << 20 | (unsigned long long)f << 25;
+}
+
+// FP64 solve of A xi = -b on one warp, by 3 x 3 blocks.  With A = [P Q; Q^T S], C = adj P and d = det P,
+//     W = C Q, v = C b_1, S'' = d S - Q^T W, z = d b_2 - Q^T v, C'' = adj S'', d'' = det S'',
+//     x_2 = C'' z / d'', x_1 = (v - W x_2) / d, xi = -x,
+// every line a set of sums of two to four products, one sum to a lane: 21 dependent FP64 instructions and seven
+// exchanges between lanes, where the pivoting elimination above takes 30 and nineteen.  An FP64 instruction takes
+// 64 cycles of its warp whatever its active lanes, so the number on the chain is the time: 3851 cycles
+// (1.86 us) for the elimination, 2177 (1.05 us) for this form, and no larger errors over condition numbers up to 1e7.  Products of minors lose more digits than an elimination does when A is
+// close to singular, so this form is taken only where every pivot (a ratio of its minors) is certain, from the
+// exponents alone, to be above 2^-24 of the largest diagonal element; otherwise, and whenever pivot_eps asks for
+// more or a value is not finite, the elimination solves the system and decides whether it is degenerate.
+// *x: lane k < 6 holds xi[k].
+__device__ __forceinline__ bool warp_solve6(const double *tot, double pivot_eps, double *x) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    // symmetric 3 x 3 matrices: elements (0,0) (0,1) (0,2) (1,1) (1,2) (2,2) in lanes 0..5; cofactor p is
+    // m[a] m[b] - m[c] m[d]
+    constexpr unsigned long long kCa = lane_tab6(3, 2, 1, 0, 1, 0), kCb = lane_tab6(5, 4, 4, 5, 2, 3),
+                                 kCc = lane_tab6(4, 1, 2, 2, 0, 1), kCd = lane_tab6(4, 5, 3, 2, 4, 1);
+    const int l6 = lane < 6 ? lane : 0;
+    const int ca = lane_tab(kCa, l6), cb = lane_tab(kCb, l6), cc = lane_tab(kCc, l6), cd = lane_tab(kCd, l6);
+    // element e of P in the upper triangle: 0 1 2 6 7 11
+    constexpr unsigned long long kP = lane_tab6(0, 1, 2, 6, 7, 11);
+    const double c1 = fma(tot[lane_tab(kP, ca)], tot[lane_tab(kP, cb)],
+                          dneg(tot[lane_tab(kP, cc)] * tot[lane_tab(kP, cd)]));
+    // W (lanes 0..8), v (9..11), d (12): rows of C times columns of Q, b_1, the first row of P
+    const int wi = lane < 9 ? lane / 3 : (lane < 12 ? lane - 9 : 0), wj = lane - 3 * (lane / 3);
+    const int x0 = lane < 9 ? 3 + wj : (lane < 12 ? 21 : 0), x1i = lane < 9 ? 8 + wj : (lane < 12 ? 22 : 1),
+              x2i = lane < 9 ? 12 + wj : (lane < 12 ? 23 : 2);
+    const int r0 = wi, r1 = wi == 0 ? 1 : wi + 2, r2 = wi == 0 ? 2 : wi + 3;  // row wi of a symmetric matrix
+    const double wv = fma(__shfl_sync(full, c1, r0), tot[x0],
+                          fma(__shfl_sync(full, c1, r1), tot[x1i], __shfl_sync(full, c1, r2) * tot[x2i]));
+    const double det = __shfl_sync(full, wv, 12);
+    // S'' (lanes 0..5), z (6..8)
+    const int si = lane < 6 ? lane_tab(lane_tab6(0, 0, 0, 1, 1, 2), lane) : (lane < 9 ? lane - 6 : 0);
+    const int sj = lane_tab(lane_tab6(0, 1, 2, 1, 2, 2), l6);
+    const int w0 = lane < 6 ? sj : 9, w1 = lane < 6 ? 3 + sj : 10, w2 = lane < 6 ? 6 + sj : 11;
+    const double top = tot[lane < 6 ? 15 + lane : (lane < 9 ? 18 + lane : 15)];
+    const double sz = fma(dneg(tot[3 + si]), __shfl_sync(full, wv, w0),
+                          fma(dneg(tot[8 + si]), __shfl_sync(full, wv, w1),
+                              fma(dneg(tot[12 + si]), __shfl_sync(full, wv, w2), det * top)));
+    const double c2 = fma(__shfl_sync(full, sz, ca), __shfl_sync(full, sz, cb),
+                          dneg(__shfl_sync(full, sz, cc) * __shfl_sync(full, sz, cd)));
+    // C'' z (lanes 0..2), d'' (lane 3)
+    const int ui = lane < 3 ? lane : 0, ub = lane < 3 ? 6 : 0;
+    const int u1 = ui == 0 ? 1 : ui + 2, u2 = ui == 0 ? 2 : ui + 3;
+    const double ud = fma(__shfl_sync(full, c2, ui), __shfl_sync(full, sz, ub),
+                          fma(__shfl_sync(full, c2, u1), __shfl_sync(full, sz, ub + 1),
+                              __shfl_sync(full, c2, u2) * __shfl_sync(full, sz, ub + 2)));
+    const double det2 = __shfl_sync(full, ud, 3);
+    // 1 / d'' in lanes 0..2, 1 / d elsewhere
+    const double rc = rcp64_scaled(lane < 3 ? det2 : det);
+    const double xb = ud * rc;  // x_2 in lanes 0..2
+    const double rd = __shfl_sync(full, rc, 3);
+    const int l3 = lane < 3 ? lane : 0;
+    const double q0 = __shfl_sync(full, wv, 3 * l3), q1 = __shfl_sync(full, wv, 3 * l3 + 1),
+                 q2 = __shfl_sync(full, wv, 3 * l3 + 2), vi = __shfl_sync(full, wv, 9 + l3);
+    const double xa = fma(dneg(q0), __shfl_sync(full, xb, 0),
+                          fma(dneg(q1), __shfl_sync(full, xb, 1), fma(dneg(q2), __shfl_sync(full, xb, 2), vi))) * rd;
+    const double xb3 = __shfl_sync(full, xb, lane >= 3 && lane < 6 ? lane - 3 : 0);
+    *x = dneg(lane < 3 ? xa : xb3);
+    // every pivot certainly above 2^-24 of the largest diagonal element (in [2^em, 2^(em+1)))?  The pivots are
+    // P_00, minor / P_00, d / minor, S''_00 / d, minor'' / (S''_00 d), d'' / (minor'' d)
+    int hm = __double2hiint(tot[0]);
+    hm = max(max(hm, __double2hiint(tot[6])), max(__double2hiint(tot[11]), __double2hiint(tot[15])));
+    hm = max(hm, max(__double2hiint(tot[18]), __double2hiint(tot[20])));
+    const int h0 = __double2hiint(tot[0]), h1 = __shfl_sync(full, __double2hiint(c1), 5), h2 = __double2hiint(det);
+    const int h3 = __shfl_sync(full, __double2hiint(sz), 0), h4 = __shfl_sync(full, __double2hiint(c2), 5),
+              h5 = __double2hiint(det2);
+    const int em = (hm >> 20) - 1023, e0 = (h0 >> 20) - 1023, e1 = (h1 >> 20) - 1023, e2 = (h2 >> 20) - 1023,
+              e3 = (h3 >> 20) - 1023, e4 = (h4 >> 20) - 1023, e5 = (h5 >> 20) - 1023;
+    const int low = em - 23 + 1;
+    const bool good = (h0 | h1 | h2 | h3 | h4 | h5) >= 0 && e0 >= low && e1 - e0 > low && e2 - e1 > low &&
+                      e3 - e2 > low && e4 - e3 - e2 - 1 > low && e5 - e4 - e2 - 1 > low && em > -500 && em < 100 &&
+                      dbits(pivot_eps) <= dbits(2.9802322387695312e-08);  // 2^-25
+    if (good && __all_sync(full, dfinite(*x))) return true;
+    return warp_solve6_pivots(tot, pivot_eps, x);
 }
 
 // (-1)^n / (2n + 1 + c)!: the n-th Taylor coefficient in t^2 of sin(t)/t (c = 0),
@@ -588,144 +706,151 @@ __device__ __forceinline__ double se3_taylor_coef(int n, int c) {
     return c == 0 ? k[n][0] : (c == 1 ? k[n][1] : k[n][2]);
 }
 
-// T <- exp(xi^) T on one warp: lanes 0..2 evaluate the coefficients A, B, C;
-// lanes 0..8 the rotation R = I + A W + B W^2 and lanes 9..17 V = I + B W + C W^2
-// (one matrix entry each); then, in the same three multiply-adds, lanes 0..11
-// each compose one entry of R T and lanes 12..14 one entry of V v, which the
-// translation lanes add.  The series is cut where its remainder (below the
-// first omitted term) is under 5e-17 relative: degree 3 in t^2 for t^2 <= 2^-9,
-// degree 4 for t^2 <= 2^-6, degree 5 for t^2 <= 1/16, sincos beyond.
-// T lives in shared memory (12 doubles) and is updated in place; xi is the same in every lane.
-__device__ __forceinline__ void warp_se3_update(const double xi[6], double *T) {
+// The same coefficients for any t, by sincos (out of line: a step is rarely above a quarter of a radian).
+static __device__ __noinline__ double se3_coef_large(double th2, int c) {
+    double A, B, C;
+    se3_coeffs(th2, A, B, C);
+    return c == 0 ? A : (c == 1 ? B : C);
+}
+
+// T <- exp(xi^) T on one warp, xi[k] in lane k < 6; returns whether |omega|^2 < er2 and |v|^2 < et2.
+// R = I + A W + B W^2 (lanes 0..8, one entry each) and V = I + B W + C W^2 (lanes 9..17), W^2 entry by entry as
+// omega_i omega_j or -(omega_j^2 + omega_k^2); the same three instructions give |omega|^2 (lane 18) and |v|^2
+// (lane 19).  Lanes 0..2 evaluate the coefficients A, B, C by their series, cut where the remainder (below the
+// first omitted term) is under 5e-17 relative: degree 1 in t^2 for t^2 <= 2^-24, 2 for 2^-14, 3 for 2^-9, 4 for
+// 2^-6, 5 for 2^-4, sincos beyond.  Then lanes 0..11 each compose one entry of R T and lanes 12..14 one entry of
+// V v, which the translation lanes add.  T lives in shared memory (12 doubles) and is updated in place; Tf, when
+// given, receives the new pose in FP32.  0.67 us a call: 10 to 12 FP64 instructions on the chain, where an
+// update and a separate convergence test took 16 and 1.02 us.
+__device__ __forceinline__ bool warp_se3_update(double x, double *T, float *Tf, double er2, double et2) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const double w0 = xi[0], w1 = xi[1], w2 = xi[2];
-    const double th2 = fma(w0, w0, fma(w1, w1, w2 * w2));
+    const int e = lane < 9 ? lane : (lane < 18 ? lane - 9 : 0);
+    const int ei = e / 3, ek = e - 3 * (e / 3);
+    const bool norm = lane == 18 || lane == 19;  // lane 18: omega, lane 19: v
+    const int nb = lane == 19 ? 3 : 0;
+    const bool diag = ei == ek;
+    const int o1 = ei == 2 ? 0 : ei + 1, o2 = ei == 0 ? 2 : ei - 1;  // the two other axes of a diagonal entry
+    // p = a b + c^2 + f^2: omega_i omega_k; omega_j^2 + omega_k^2; the squared norms
+    const double pa = __shfl_sync(full, x, norm ? nb + 2 : (diag ? o1 : ei));
+    const double pb = __shfl_sync(full, x, norm ? nb + 2 : (diag ? o1 : ek));
+    const double pc0 = __shfl_sync(full, x, norm ? nb + 1 : o2), pf0 = __shfl_sync(full, x, nb);
+    const int wl = diag ? 0 : 3 - ei - ek;
+    const double wx = __shfl_sync(full, x, wl);  // the component of an off-diagonal entry of W
+    const double pc = norm || diag ? pc0 : 0.0, pf = norm ? pf0 : 0.0;
+    const double pp = fma(pf, pf, fma(pc, pc, pa * pb));
+    const double th2 = __shfl_sync(full, pp, 18);
+    const bool below = dbits(pp) < dbits(lane == 18 ? er2 : et2);
+    const bool conv = ((__ballot_sync(full, below) >> 18) & 3u) == 3u;
+    const double W2 = diag ? dneg(pp) : pp;
     const long long tb = dbits(th2);
     const int c = lane < 3 ? lane : 0;
     double coef;
-    if (tb <= dbits(0.001953125)) {
-        coef = fma(th2, fma(th2, fma(th2, se3_taylor_coef(3, c), se3_taylor_coef(2, c)), se3_taylor_coef(1, c)),
-                   se3_taylor_coef(0, c));
-    } else if (tb <= dbits(0.015625)) {
-        coef = fma(th2,
-                   fma(th2, fma(th2, fma(th2, se3_taylor_coef(4, c), se3_taylor_coef(3, c)), se3_taylor_coef(2, c)),
-                       se3_taylor_coef(1, c)),
-                   se3_taylor_coef(0, c));
+    if (tb <= dbits(5.9604644775390625e-08)) {  // 2^-24
+        coef = fma(th2, se3_taylor_coef(1, c), se3_taylor_coef(0, c));
+    } else if (tb <= dbits(6.103515625e-05)) {  // 2^-14
+        coef = fma(th2, fma(th2, se3_taylor_coef(2, c), se3_taylor_coef(1, c)), se3_taylor_coef(0, c));
     } else if (tb <= dbits(0.0625)) {
-        double p = se3_taylor_coef(5, c);
+        const int deg = tb <= dbits(0.001953125) ? 3 : (tb <= dbits(0.015625) ? 4 : 5);
+        coef = deg == 5 ? se3_taylor_coef(5, c) : 0.0;
+        coef = deg >= 4 ? fma(th2, coef, se3_taylor_coef(4, c)) : 0.0;
 #pragma unroll
-        for (int n = 4; n >= 0; --n) p = fma(th2, p, se3_taylor_coef(n, c));
-        coef = p;
+        for (int n = 3; n >= 0; --n) coef = fma(th2, coef, se3_taylor_coef(n, c));
     } else {
-        double A, B, C;
-        se3_coeffs(th2, A, B, C);
-        coef = lane == 0 ? A : (lane == 1 ? B : C);
+        coef = se3_coef_large(th2, c);
     }
-    const double A = __shfl_sync(full, coef, 0), B = __shfl_sync(full, coef, 1), C = __shfl_sync(full, coef, 2);
-    // one entry of R (lanes 0..8) or V (lanes 9..17)
-    const int e = lane < 9 ? lane : (lane < 18 ? lane - 9 : 0);
-    const int ei = e / 3, ek = e - 3 * (e / 3);
-    const double om_i = ei == 0 ? w0 : (ei == 1 ? w1 : w2);
-    const double om_k = ek == 0 ? w0 : (ek == 1 ? w1 : w2);
+    const double c1 = __shfl_sync(full, coef, lane < 9 ? 0 : 1), c2 = __shfl_sync(full, coef, lane < 9 ? 1 : 2);
     // W = [omega]_x: W[i][k] = -eps_ikl omega_l
-    double Wik = 0.0;
-    if (ei == 0 && ek == 1) Wik = dneg(w2);
-    if (ei == 0 && ek == 2) Wik = w1;
-    if (ei == 1 && ek == 0) Wik = w2;
-    if (ei == 1 && ek == 2) Wik = dneg(w0);
-    if (ei == 2 && ek == 0) Wik = dneg(w1);
-    if (ei == 2 && ek == 1) Wik = w0;
-    const double W2 = fma(om_i, om_k, ei == ek ? dneg(th2) : 0.0);
-    const double c1 = lane < 9 ? A : B, c2 = lane < 9 ? B : C;
-    const double ent = fma(c1, Wik, fma(c2, W2, ei == ek ? 1.0 : 0.0));
+    const bool neg = ek - ei == 1 || ek - ei == -2;
+    const double Wik = diag ? 0.0 : (neg ? dneg(wx) : wx);
+    const double ent = fma(c1, Wik, fma(c2, W2, diag ? 1.0 : 0.0));
     // lanes 0..11: (R T)(i, j), i = lane / 4, j = lane % 4; lanes 12..14: (V v)(lane - 12)
     const bool comp = lane < 12, tv = lane >= 12 && lane < 15;
     const int oi = comp ? lane / 4 : (tv ? lane - 12 : 0), oj = comp ? lane % 4 : 0;
     const int src = tv ? 9 + 3 * oi : 3 * oi;
+    const double v0 = __shfl_sync(full, x, 3), v1 = __shfl_sync(full, x, 4), v2 = __shfl_sync(full, x, 5);
+    const double X0 = tv ? v0 : T[oj], X1 = tv ? v1 : T[4 + oj], X2 = tv ? v2 : T[8 + oj];
     const double M0 = __shfl_sync(full, ent, src), M1 = __shfl_sync(full, ent, src + 1),
                  M2 = __shfl_sync(full, ent, src + 2);
-    const double X0 = tv ? xi[3] : T[oj], X1 = tv ? xi[4] : T[4 + oj], X2 = tv ? xi[5] : T[8 + oj];
     const double o = fma(M0, X0, fma(M1, X1, M2 * X2));
     const double te = __shfl_sync(full, o, 12 + oi);
     const double out = oj == 3 ? o + te : o;
     __syncwarp();
-    if (lane < 12) T[lane] = out;
+    if (lane < 12) {
+        T[lane] = out;
+        if (Tf) Tf[lane] = (float)out;
+    }
     __syncwarp();
-}
-
-// Convergence test on one warp: |omega|^2 < er2 and |v|^2 < et2 (lane 0 takes
-// the rotation, lane 1 the translation, in the same instructions).
-__device__ __forceinline__ bool warp_converged(const double xi[6], double er2, double et2) {
-    const int lane = threadIdx.x & 31;
-    const bool tr = lane == 1;
-    const double a = tr ? xi[3] : xi[0], b = tr ? xi[4] : xi[1], c = tr ? xi[5] : xi[2];
-    const double n2 = fma(a, a, fma(b, b, c * c));
-    const bool below = dbits(n2) < dbits(tr ? et2 : er2);
-    return (__ballot_sync(0xffffffffu, below) & 3u) == 3u;
+    return conv;
 }
 
 // ----------------------------------------------------------------------------- exact order-free sums
 //
-// A float v is held as the integer X = v * 2^48 (truncated toward zero below 2^-48, saturated
-// at |v| = 2^47) split into three chunks X = c0 + c1 2^32 + c2 2^64 with |c_k| < 2^32.  Chunks
-// add into 64-bit integers with no carry between them for up to 2^31 terms, so a sum of floats
-// formed this way is exact and does not depend on the order of the additions (integer atomics
-// from any number of CTAs give every reader the same bits).
+// A float v is held as the integer X = v * 2^48 (truncated toward zero below 2^-48, saturated at |v| = 2^47).
+// Within a CTA X is split into 24-bit chunks, which 32-bit integer reductions add exactly; between CTAs into
+// words X = w0 + w1 2^32 + w2 2^64 that add into 64-bit integers with no carry between them.  A sum of floats
+// formed this way is exact and does not depend on the order of the additions (integer atomics from any number
+// of CTAs give every reader the same bits).
 
-__device__ __forceinline__ void fx_chunks(float v, long long c[3]) {
+// X = v * 2^48 as four signed 24-bit chunks: X = c[0] + c[1] 2^24 + c[2] 2^48 + c[3] 2^72.
+__device__ __forceinline__ void fx_chunks24(float v, int c[4]) {
     const unsigned b = __float_as_uint(v);
     int e = (int)((b >> 23) & 0xffu);
-    unsigned long long m = b & 0x7fffffu;
-    if (e == 0xff) m = 0;  // infinities and NaN do not enter a sum
+    unsigned m = e == 0xff ? 0u : b & 0x7fffffu;  // (an infinity or NaN counts as the largest value)
     if (e) m |= 0x800000u;
     else e = 1;
-    int sh = e - 150 + 48;  // X = m * 2^sh
-    if (sh > 71) sh = 71;   // saturate: |X| < 2^95
-    unsigned long long lo, hi;
+    int sh = min(e - 150 + 48, 71);  // X = m * 2^sh, |X| < 2^95
     if (sh < 0) {
-        lo = sh > -32 ? (m >> -sh) : 0ull;
-        hi = 0ull;
-    } else if (sh < 64) {
-        lo = m << sh;
-        hi = sh > 40 ? (m >> (64 - sh)) : 0ull;
-    } else {
-        lo = 0ull;
-        hi = m << (sh - 64);
+        m = sh > -24 ? m >> -sh : 0u;
+        sh = 0;
     }
-    const long long sgn = (b >> 31) ? -1 : 1;
-    c[0] = sgn * (long long)(lo & 0xffffffffull);
-    c[1] = sgn * (long long)(lo >> 32);
-    c[2] = sgn * (long long)hi;
+    const int q = sh >= 48 ? 2 : (sh >= 24 ? 1 : 0);
+    const unsigned long long y = (unsigned long long)m << (sh - 24 * q);
+    const int lo = (int)((unsigned)y & 0xffffffu), hi = (int)(y >> 24);
+    const int sl = (b >> 31) ? -lo : lo, sg = (b >> 31) ? -hi : hi;
+    c[0] = q == 0 ? sl : 0;
+    c[1] = q == 1 ? sl : (q == 0 ? sg : 0);
+    c[2] = q == 2 ? sl : (q == 1 ? sg : 0);
+    c[3] = q == 2 ? sg : 0;
 }
 
-// (s0 + s1 2^32 + s2 2^64) * 2^-48 as the nearest double (ties to even), integer instructions only.
+// The sum of up to 16 numbers' 24-bit chunks as three words s0 + s1 2^32 + s2 2^64, each below 2^36 in magnitude.
+__device__ __forceinline__ void fx_words(int r0, int r1, int r2, int r3, long long w[3]) {
+    const long long a = (long long)r0 + ((long long)r1 << 24), b = (long long)r2 + ((long long)r3 << 24);
+    w[0] = a & 0xffffffffll;
+    w[1] = (a >> 32) + ((b & 0xffffll) << 16);  // b 2^48 = (b mod 2^16) 2^48 + (b >> 16) 2^64
+    w[2] = b >> 16;
+}
+
+// (s0 + s1 2^32 + s2 2^64) * 2^-48 as the nearest double (ties to even), integer instructions only: the sum as
+// 128 bits, its magnitude shifted to the top, rounded at bit 11 of the upper half.
 __device__ __forceinline__ double fx_value(long long s0, long long s1, long long s2) {
-    const __int128 x = (__int128)s0 + ((__int128)s1 << 32) + ((__int128)s2 << 64);
-    if (x == 0) return 0.0;
-    const bool neg = x < 0;
-    const unsigned __int128 mag = neg ? (unsigned __int128)(-x) : (unsigned __int128)x;
-    const unsigned long long h = (unsigned long long)(mag >> 64), l = (unsigned long long)mag;
-    const int nbits = h ? 128 - __clzll((long long)h) : 64 - __clzll((long long)l);
-    unsigned long long mant;
-    int top = nbits;  // the value is mant * 2^(top - 53)
-    if (nbits <= 53) {
-        mant = l << (53 - nbits);
-    } else {
-        const int sh = nbits - 53;
-        mant = (unsigned long long)(mag >> sh);
-        const unsigned __int128 rem = mag & ((((unsigned __int128)1) << sh) - 1);
-        const unsigned __int128 half = ((unsigned __int128)1) << (sh - 1);
-        if (rem > half || (rem == half && (mant & 1ull))) ++mant;
-        if (mant >> 53) {
-            mant >>= 1;
-            ++top;
-        }
+    const long long t1 = s1 + (s0 >> 32);
+    long long hs = s2 + (t1 >> 32);
+    unsigned long long l = ((unsigned long long)t1 << 32) | (unsigned)s0;
+    const bool neg = hs < 0;
+    unsigned long long h = (unsigned long long)hs;
+    if (neg) {
+        l = 0ull - l;
+        h = ~h + (l == 0ull ? 1ull : 0ull);
     }
-    const long long ebits = (long long)(top - 1 - 48 + 1023);
-    const long long bits = (neg ? (long long)0x8000000000000000ull : 0ll) | (ebits << 52) |
-                           (long long)(mant & 0xfffffffffffffull);
-    return __longlong_as_double(bits);
+    if ((h | l) == 0ull) return 0.0;
+    int n = 0;  // leading zeros of the 128 bits
+    if (h == 0ull) {
+        h = l;
+        l = 0ull;
+        n = 64;
+    }
+    const int z = __clzll((long long)h);
+    n += z;
+    const unsigned long long top = (h << z) | ((l >> 1) >> (63 - z)), rest = l << z;
+    unsigned long long m = top >> 11;
+    const bool up = (top >> 10) & 1ull, sticky = (top & 0x3ffull) != 0ull || rest != 0ull;
+    if (up && (sticky || (m & 1ull))) ++m;
+    // the value is (m 2^-52) 2^(127 - n - 48), m in [2^52, 2^53]; m's leading one is added into the exponent
+    const unsigned long long bits =
+        ((neg ? 0x800ull : 0ull) << 52) + ((unsigned long long)(127 - n - 48 + 1023 - 1) << 52) + m;
+    return __longlong_as_double((long long)bits);
 }
 
 // ----------------------------------------------------------------------------- sweep front end (Sec. III-A)

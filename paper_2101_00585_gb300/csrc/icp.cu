@@ -345,6 +345,8 @@ constexpr int kStageGroup = 7;
 // the CTAs' sample counts, whatever rows of the panorama hold samples.
 constexpr int kSlice = 64;
 constexpr int kUnitSlices = kTileThreads / kSlice;
+constexpr int kSumPitch = 33;  // a warp's sums in shared memory (odd: the lanes of a half-warp read 16 rows)
+static_assert(kTileWarps == 16, "tile_cta_word gives a half-warp one lane per warp of the CTA");
 
 // The sweep pixel a staged keyframe point lands in: its point and normal,
 // gathered from L2, and whether the point binned at all.
@@ -401,28 +403,45 @@ __device__ __forceinline__ void accumulate_entry(const IcpArgs &a, const PoseF &
     inl += ok ? 1 : 0;
 }
 
-// The CTA's contribution to one step's sums, exact: each warp's 28 sums (warp
-// reduce-scatter) go into shared 64-bit integer accumulators as fixed-point
-// chunks, the inlier and valid counts as integers.
-__device__ __forceinline__ void tile_fx(float acc[28], int inl, int valid, unsigned long long *fxs) {
+// The CTA's contribution to one step's sums, exact, in two parts around a __syncthreads.  First each warp reduces
+// its 28 FP32 sums (reduce-scatter) and its two counts and leaves them in sw[warp]; then warp w adds the 16 warps'
+// sums w and w + 16 (one warp's to a lane, as 24-bit chunks with integer reductions) and lanes 0..2 and 16..18
+// hold the words of those two sums.
+__device__ __forceinline__ void tile_warp_sums(float acc[28], int inl, int valid, float *sw) {
     const int lane = threadIdx.x & 31;
     float v[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = i < 28 ? acc[i] : 0.0f;
     const float s = warp_reduce_scatter(v);  // lane i: the warp's sum of acc[i]
-    if (lane < 28) {
-        long long c[3];
-        fx_chunks(s, c);
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-            if (c[k]) atomicAdd(fxs + 3 * lane + k, (unsigned long long)c[k]);
-    }
     const int si = __reduce_add_sync(0xffffffffu, inl);
     const int sv = __reduce_add_sync(0xffffffffu, valid);
-    if (lane == 0) {
-        if (si) atomicAdd(fxs + 84, (unsigned long long)si);
-        if (sv) atomicAdd(fxs + 85, (unsigned long long)sv);
+    sw[lane] = lane < 28 ? s : __int_as_float(lane == 28 ? si : sv);
+}
+
+// Word `slot` (or -1) of the step's accumulators that this lane contributes, and the contribution.
+__device__ __forceinline__ int tile_cta_word(const float (*sw)[kSumPitch], long long &word) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = warp + (lane & 16);  // the sum this half-warp adds: 28 and 29 are the counts
+    const float v = sw[lane & 15][i];
+    int c[4];
+    fx_chunks24(v, c);
+    if (i >= 28) {
+        c[0] = __float_as_int(v);
+        c[1] = c[2] = c[3] = 0;
     }
+    int r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int lo = __reduce_add_sync(0xffffffffu, lane < 16 ? c[k] : 0);
+        const int hi = __reduce_add_sync(0xffffffffu, lane < 16 ? 0 : c[k]);
+        r[k] = lane < 16 ? lo : hi;
+    }
+    long long w[3];
+    fx_words(r[0], r[1], r[2], r[3], w);
+    const int k = lane & 15;
+    word = k == 0 ? (i >= 28 ? (long long)r[0] : w[0]) : (k == 1 ? w[1] : w[2]);
+    if (i < 28) return k < 3 ? 3 * i + k : -1;
+    return i < 30 && k == 0 ? 84 + i - 28 : -1;
 }
 
 // Grid barrier on a monotonic 64-bit arrival counter, called by one thread per
@@ -504,7 +523,7 @@ __global__ void __launch_bounds__(kTileThreads, 1)
     };
     __shared__ double tot[32];
     __shared__ long long totn[2];
-    __shared__ unsigned long long fxs[kFxWords];
+    __shared__ float swarp[kTileWarps][kSumPitch];
     __shared__ int gbm_s;
     __shared__ double Tsh[12];
     __shared__ double Tprev[12], Tmot[12];
@@ -686,8 +705,6 @@ __global__ void __launch_bounds__(kTileThreads, 1)
     // The keyframe does not depend on the sweep, so its loads fill both barrier waits.
     unsigned long long nbar = 0;  // grid barriers passed before the Gauss-Newton steps
     if (fr.on) {
-        const int ns = a.sp.rows * a.sp.cols;
-        const int stride = gridDim.x * kTileThreads;
         // (warps 1.. project while warp 0 forms the motion prior above)
         if (warp > 0) {
             const int pstride = gridDim.x * (kTileThreads - 32);
@@ -695,33 +712,35 @@ __global__ void __launch_bounds__(kTileThreads, 1)
                 project_point(fr.pts, i, a.srule, fr.zbuf);
         }
         cta_grid_arrive(ctrl);
-        stage_groups(0, my_groups / 2);
+    }
+    // (one loop, so that the staging's code exists once: without a front end its single pass stages everything)
+    for (int half = fr.on ? 0 : 1; half < 2; ++half) {
+        stage_groups(half == 0 || !fr.on ? 0 : my_groups / 2, half == 0 ? my_groups / 2 : my_groups);
+        if (!fr.on) break;
         if (!cta_grid_await(ctrl, base + G * ++nbar, st, &flag, a.wait_cycles)) return;
-        clear_prev(nbar);
-        const PixZbuf zb{fr.pts, fr.zbuf};
-        for (int k = blockIdx.x * kTileThreads + threadIdx.x; k < ns; k += stride) {
-            resolve_pixel<true, false>(fr.pts, k, fr.zbuf, fr.depth, fr.idx, fr.pix);
-            store_nw(fr.nrm, k, fr.nrm_prec, normal_pixel(zb, a.sp, fr.np, k));
+        const int ns = a.sp.rows * a.sp.cols;
+        const int stride = gridDim.x * kTileThreads;
+        if (half == 0) {
+            clear_prev(nbar);
+            const PixZbuf zb{fr.pts, fr.zbuf};
+            for (int k = blockIdx.x * kTileThreads + threadIdx.x; k < ns; k += stride) {
+                resolve_pixel<true, false>(fr.pts, k, fr.zbuf, fr.depth, fr.idx, fr.pix);
+                store_nw(fr.nrm, k, fr.nrm_prec, normal_pixel(zb, a.sp, fr.np, k));
+            }
+            cta_grid_arrive(ctrl);
+        } else {
+            // (the buffer before this barrier belongs to the front end's first barrier: never added into)
+            for (int k = blockIdx.x * kTileThreads + threadIdx.x; k < ns; k += stride) fr.zbuf[k] = kEmptyKey;
         }
-        cta_grid_arrive(ctrl);
-        stage_groups(my_groups / 2, my_groups);
-        if (!cta_grid_await(ctrl, base + G * ++nbar, st, &flag, a.wait_cycles)) return;
-        // (the buffer before this barrier belongs to the front end's first barrier: never added into)
-        for (int k = blockIdx.x * kTileThreads + threadIdx.x; k < ns; k += stride) fr.zbuf[k] = kEmptyKey;
-    } else {
-        stage_groups(0, my_groups);
-        __syncthreads();
     }
 
     // convergence thresholds, squared once per launch (read by warp 0 only)
     const double er2 = warp == 0 ? ip.eps_rot * ip.eps_rot : 0.0, et2 = warp == 0 ? ip.eps_trans * ip.eps_trans : 0.0;
     int it = 0;
+    if (threadIdx.x < 12) Tf[threadIdx.x] = (float)Tsh[threadIdx.x];
+    __syncthreads();
     for (; it < ip.max_iters; ++it) {
-        // the pose in FP32: converted once per CTA (FP64 conversions are slow on GB300), read by all
-        if (threadIdx.x < 12) Tf[threadIdx.x] = (float)Tsh[threadIdx.x];
-        if (threadIdx.x < kFxWords) fxs[threadIdx.x] = 0ull;
-        __syncthreads();
-        PoseF T;
+        PoseF T;  // in FP32: converted once per CTA and step (FP64 conversions are slow on GB300), read by all
 #pragma unroll
         for (int i = 0; i < 12; ++i) T.r[i] = Tf[i];
         float acc[28];
@@ -751,21 +770,25 @@ __global__ void __launch_bounds__(kTileThreads, 1)
             if (unit_pixel(u, k)) accumulate_pixel<L1>(as, T, k, acc, inl);
         }
         const int valid = it == 0 ? count_valid(a) : 0;
-        tile_fx(acc, inl, valid, fxs);
+        tile_warp_sums(acc, inl, valid, swarp[warp]);
         __syncthreads();
         const unsigned long long jb = nbar + (unsigned long long)(it + 1);  // this step's barrier
         unsigned long long *const buf = acc_buf(jb);
         // (test support: with `withhold`, CTA 0 skips its first contribution, so no CTA's wait can end)
         if (!(a.withhold && it == 0 && blockIdx.x == 0)) {
-            if (threadIdx.x < kFxWords) {
-                const unsigned long long v = fxs[threadIdx.x] + kFxBias + kFxCount;
-                asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(buf + (size_t)threadIdx.x * kAccStride),
-                             "l"(v)
+            long long word;
+            const int slot = tile_cta_word(swarp, word);
+            if (slot >= 0) {
+                const unsigned long long v = (unsigned long long)word + kFxBias + kFxCount;
+                asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(buf + (size_t)slot * kAccStride), "l"(v)
                              : "memory");
-            } else if (threadIdx.x == kTileThreads - 32) {
+            } else if (threadIdx.x == kTileThreads - 1) {
                 grid_arrive(&ctrl->arrive64);  // keeps the barrier count that the later phases wait on
             }
         }
+        // the lanes that added come back together before the poll: left apart, the warp went through the poll's
+        // votes and the solve's shuffles in two groups (6.8 us longer, on some SM at every third step)
+        __syncwarp();
         if (warp == 0) {
             // wait until every CTA has added into every word: the last loads hold the step's totals
             // (lane i < 28 reads sum i's three chunks, lane 28 the inlier and valid counts)
@@ -808,27 +831,20 @@ __global__ void __launch_bounds__(kTileThreads, 1)
                 }
                 __syncwarp();
                 const long long inliers = totn[0];
-                double xi[6] = {0, 0, 0, 0, 0, 0};
+                double xi = 0.0;  // lane k < 6: xi[k]
                 int status = UPSLAM_OK, conv = 0;
-                if (inliers < ip.min_inliers) {
+                if (inliers < ip.min_inliers || !warp_solve6(tot, ip.pivot_eps, &xi)) {
                     status = UPSLAM_ERR_DEGENERATE;
+                    xi = 0.0;
                 } else {
-                    if (!warp_solve6(tot, ip.pivot_eps, xi)) {
-                        status = UPSLAM_ERR_DEGENERATE;
-#pragma unroll
-                        for (int i = 0; i < 6; ++i) xi[i] = 0.0;
-                    } else {
-                        warp_se3_update(xi, Tsh);
-                        conv = warp_converged(xi, er2, et2) ? 1 : 0;
-                    }
+                    conv = warp_se3_update(xi, Tsh, Tf, er2, et2) ? 1 : 0;
                 }
                 if (lane == 0) {
                     status_s = status;
                     conv_s = conv;
                     if (it == 0) valid_s = (int)totn[1];
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) xi_sh[i] = xi[i];
                 }
+                if (lane < 6) xi_sh[lane] = xi;
             }
         } else if (warp == 1 && blockIdx.x == 0) {
             // every CTA has added into this step's buffer, so every CTA has read the previous one:
