@@ -27,7 +27,6 @@ namespace upslam {
 
 struct ConsSide {
     upslam_pano pp;
-    BinRule rule;
     float *depth;
     void *nw;
     int prec;
@@ -67,7 +66,7 @@ __device__ __forceinline__ bool seen_through(const ConsSide &src, const ConsSide
     const float3 q = xform_inv(T, s.x, s.y, s.z);
     int jv, ju;
     float r;
-    if (!bin_pixel(q.x, q.y, q.z, dst.rule, jv, ju, r)) return false;
+    if (!bin_point(q.x, q.y, q.z, dst.pp, jv, ju, r)) return false;
     const int Wd = dst.pp.cols;
     if (!(__ldg(dst.depth + jv * Wd + ju) > 0.0f)) return false;
     const float lim = __fadd_rn(__fadd_rn(__fmul_rn(rel, r), abs_m), r);
@@ -147,8 +146,8 @@ extern "C" upslam_status upslam_keyframe_consistency(const upslam_keyframe *kf_a
         return UPSLAM_ERR_INVALID_ARG;
     if (d_removed2 && !upslam_aligned(d_removed2, 8)) return UPSLAM_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    ConsSide a{kf_a->pano, make_bin_rule(kf_a->pano), kf_a->d_depth, kf_a->d_nw, kf_a->precision, kf_a->d_dirs};
-    ConsSide b{kf_b->pano, make_bin_rule(kf_b->pano), kf_b->d_depth, kf_b->d_nw, kf_b->precision, kf_b->d_dirs};
+    ConsSide a{kf_a->pano, kf_a->d_depth, kf_a->d_nw, kf_a->precision, kf_a->d_dirs};
+    ConsSide b{kf_b->pano, kf_b->d_depth, kf_b->d_nw, kf_b->precision, kf_b->d_dirs};
     unsigned char *flags_a = reinterpret_cast<unsigned char *>(d_ws);
     unsigned char *flags_b = flags_a + align256((size_t)kf_a->pano.rows * kf_a->pano.cols);
     const int64_t na = (int64_t)kf_a->pano.rows * kf_a->pano.cols, nb = (int64_t)kf_b->pano.rows * kf_b->pano.cols;

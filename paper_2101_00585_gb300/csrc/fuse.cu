@@ -136,8 +136,6 @@ bool upslam_fuse_view(const upslam_keyframe *kf, const upslam_sweep *sw, const u
     f.kprec = kf->precision;
     f.kdirs = kf->d_dirs;
     f.sp = sw->pano;
-    f.krule = make_bin_rule(kf->pano);
-    f.srule = make_bin_rule(sw->pano);
     f.spix = reinterpret_cast<const float4 *>(sw->d_pix);
     f.snrm = sw->d_nrm;
     f.sprec = sw->nrm_precision;

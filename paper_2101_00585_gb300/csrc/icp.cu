@@ -709,7 +709,7 @@ __global__ void __launch_bounds__(kTileThreads, 1)
         if (warp > 0) {
             const int pstride = gridDim.x * (kTileThreads - 32);
             for (int i = blockIdx.x * (kTileThreads - 32) + threadIdx.x - 32; i < fr.n; i += pstride)
-                project_point(fr.pts, i, a.srule, fr.zbuf);
+                project_point(fr.pts, i, a.sp, fr.zbuf);
         }
         cta_grid_arrive(ctrl);
     }

@@ -35,11 +35,11 @@ __global__ void pano_dirs_kernel(upslam_pano pp, float *dirs) {
 
 template <bool kPose>
 __global__ void __launch_bounds__(256) project_kernel(const float4 *__restrict__ pts, int n, const double *pose,
-                                                      BinRule rule, unsigned long long *__restrict__ zbuf) {
+                                                      upslam_pano pp, unsigned long long *__restrict__ zbuf) {
     pdl_release();  // the resolve launch may place its CTAs while this grid drains
     if (!kPose) {
         for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-            project_point(pts, i, rule, zbuf);
+            project_point(pts, i, pp, zbuf);
         return;
     }
     const PoseF T = cta_pose_f32(pose);
@@ -49,9 +49,9 @@ __global__ void __launch_bounds__(256) project_kernel(const float4 *__restrict__
         const float3 q = xform(T, p.x, p.y, p.z);
         int v, u;
         float r;
-        if (!bin_pixel(q.x, q.y, q.z, rule, v, u, r)) continue;
+        if (!bin_point(q.x, q.y, q.z, pp, v, u, r)) continue;
         const unsigned long long key = ((unsigned long long)__float_as_uint(r) << 32) | (unsigned int)i;
-        atomicMin(zbuf + (size_t)v * rule.pp.cols + u, key);
+        atomicMin(zbuf + (size_t)v * pp.cols + u, key);
     }
 }
 
@@ -105,11 +105,10 @@ extern "C" upslam_status upslam_project(const float *d_pts, int32_t n, const dou
     unsigned long long *zb = reinterpret_cast<unsigned long long *>(d_zbuf);
     if (n > 0) {
         const int g = upslam_grid(n, 256);
-        const BinRule rule = make_bin_rule(*pp);
         if (d_pose12)
-            project_kernel<true><<<g, 256, 0, s>>>(reinterpret_cast<const float4 *>(d_pts), n, d_pose12, rule, zb);
+            project_kernel<true><<<g, 256, 0, s>>>(reinterpret_cast<const float4 *>(d_pts), n, d_pose12, *pp, zb);
         else
-            project_kernel<false><<<g, 256, 0, s>>>(reinterpret_cast<const float4 *>(d_pts), n, nullptr, rule, zb);
+            project_kernel<false><<<g, 256, 0, s>>>(reinterpret_cast<const float4 *>(d_pts), n, nullptr, *pp, zb);
         UPSLAM_CHECK_LAUNCH();
     }
     const int npx = pp->rows * pp->cols;
