@@ -82,15 +82,12 @@ struct BatchHit {
     bool binned;
 };
 
-__device__ __forceinline__ BatchHit batch_gather(const BatchArgs &a, const float *ent, int cap, const PoseF &Tp, int q,
-                                                 float3 &s, float3 &n) {
-    s = make_float3(ent[q], ent[cap + q], ent[2 * cap + q]);
-    n = make_float3(ent[3 * cap + q], ent[4 * cap + q], ent[5 * cap + q]);
-    const float3 qq = xform_inv(Tp, s.x, s.y, s.z);
-    int jv = 0, ju = 0;
+__device__ __forceinline__ BatchHit batch_gather(const BatchArgs &a, const PoseF &Tp, float3 s) {
+    const float3 q = xform_inv(Tp, s.x, s.y, s.z);
+    const int cell = bin_pixel(q.x, q.y, q.z, a.srule);
     BatchHit h;
-    h.binned = bin_pixel(qq.x, qq.y, qq.z, a.srule, jv, ju);
-    const int j = h.binned ? jv * a.sp.cols + ju : 0;
+    h.binned = cell >= 0;
+    const int j = cell >= 0 ? cell : 0;
     h.P = __ldg(a.spix + j);
     h.m = load_nw(a.snrm, j, a.sprec);
     return h;
@@ -134,6 +131,7 @@ __device__ __forceinline__ void batch_accumulate(const BatchArgs &a, const PoseF
     inl += ok ? 1 : 0;
 }
 
+constexpr int kAheadB = 4;  // samples of a lane binned and gathered before the first is reduced
 constexpr int kPx = 8;  // keyframe pixels per thread in flight in the prologue
 
 // Keyframe pixel k as a sample: it holds one when its depth is positive and its normal unit (the test of the
@@ -154,6 +152,8 @@ __global__ void __launch_bounds__(512, 1) icp_batched_kernel(BatchArgs a) {
     __shared__ int kf_cap[kBatchMaxKf];                      // its pixels: the length of each array
     __shared__ int kf_lo[kBatchMaxKf], kf_hi[kBatchMaxKf];   // this CTA's slice of its samples
     __shared__ int kf_wb[kBatchMaxKf];                       // where this CTA's own samples go
+    __shared__ int kf_tot[kBatchMaxKf], kf_order[kBatchMaxKf];  // samples, and the keyframes by falling samples
+    __shared__ int next_item;                                // the next work item of the step
     __shared__ int wcnt[32];
     __shared__ int pcnt[2][kPx][16];
     __shared__ int flag_s, any_active;
@@ -290,8 +290,16 @@ __global__ void __launch_bounds__(512, 1) icp_batched_kernel(BatchArgs a) {
                     tot += v;
                 }
                 kf_wb[kf] = before;
+                kf_tot[kf] = tot;
                 kf_lo[kf] = (int)((long long)tot * blockIdx.x / gridDim.x);
                 kf_hi[kf] = (int)((long long)tot * (blockIdx.x + 1) / gridDim.x);
+            }
+            __syncthreads();
+            for (int kf = threadIdx.x; kf < a.n_kf; kf += T) {
+                int rank = 0;
+                for (int o = 0; o < a.n_kf; ++o)
+                    rank += kf_tot[o] > kf_tot[kf] || (kf_tot[o] == kf_tot[kf] && o < kf) ? 1 : 0;
+                kf_order[rank] = kf;
             }
             __syncthreads();
         }
@@ -315,20 +323,25 @@ __global__ void __launch_bounds__(512, 1) icp_batched_kernel(BatchArgs a) {
         // this step's Omega distance gate (coarse-to-fine when coarse_iters > 0)
         const float gate2 = (a.ip.coarse_iters > 0 && it >= a.ip.coarse_iters) ? a.d_max2_fine : a.d_max2;
         for (int i = threadIdx.x; i < a.n_prob * kRecWords; i += T) acc[i] = 0.0f;
+        if (threadIdx.x == 0) next_item = nw;  // the first nw items are the warps' own
         __syncthreads();
         // ---- 1. accumulate.  A work item is one problem p = (keyframe kf, hypothesis h) over every
-        // sample this CTA staged for kf.  One warp takes an item (items dealt round-robin to the
-        // warps), keeps the 28 sums and the inlier count per lane in registers, reduces them once
-        // (reduce-scatter) and stores the totals to p's accumulator.  No two warps add into one
-        // accumulator, so the sums do not depend on timing.  With fewer problems than warps, `split`
-        // warps share a problem (each takes every split-th group of 32 samples) and their totals are
-        // added in warp order.  Each lane bins and gathers its next sample before it reduces the
-        // current one, so the L2 round trips overlap the arithmetic.
+        // sample this CTA staged for kf.  One warp takes an item (the next one when it is free, the
+        // keyframes with most samples first, so that the warps end together), keeps the 28 sums and the
+        // inlier count per lane in registers, reduces them once (reduce-scatter) and stores the totals to
+        // p's accumulator.  No two warps add into one accumulator, so the sums do not depend on timing or
+        // on which warp took the item.  With fewer problems than warps, `split` warps share a problem
+        // (each takes every split-th group of 32 samples) and their totals are added in part order.
+        // A lane's samples are taken kAheadB at a time: read, binned and their gathers issued together, then
+        // reduced in the same order as one by one, so that each round trip to L2 serves four samples.
         const int split = a.n_prob < nw ? nw / a.n_prob : 1;
-        for (int item = warp; item < a.n_prob * split; item += nw) {
-            const int p = item / split, part = item - p * split;
+        for (int item = warp; item < a.n_prob * split;) {
+            const int w = item / split, part = item - w * split;  // the w-th problem in that order
+            const int kf = kf_order[w / a.n_hyp], p = kf * a.n_hyp + w % a.n_hyp;
+            int nx = 0;
+            if (lane == 0) nx = atomicAdd(&next_item, 1);
+            item = __shfl_sync(0xffffffffu, nx, 0);
             if (!act[p]) continue;
-            const int kf = p / a.n_hyp;
             const int lo = kf_lo[kf], hi = kf_hi[kf], capk = kf_cap[kf];
             const float *E = a.entries + kf_base[kf];
             PoseF Tp;
@@ -340,18 +353,24 @@ __global__ void __launch_bounds__(512, 1) icp_batched_kernel(BatchArgs a) {
             int inl = 0;
             const int stride = 32 * split;
             int e = lo + part * 32 + lane;
-            if (e < hi) {
-                float3 sc, nc;
-                BatchHit hc = batch_gather(a, E, capk, Tp, e, sc, nc);
-                for (; e < hi; e += stride) {
-                    float3 sn = sc, nn = nc;
-                    BatchHit hn = hc;
-                    if (e + stride < hi) hn = batch_gather(a, E, capk, Tp, e + stride, sn, nn);
-                    batch_accumulate(a, Tp, gate2, sc, nc, hc, accr, inl);
-                    sc = sn;
-                    nc = nn;
-                    hc = hn;
+            for (; e < hi; e += kAheadB * stride) {
+                // (past the end the last sample is taken again and not used)
+                int q[kAheadB];
+                float3 s[kAheadB], n[kAheadB];
+                BatchHit h[kAheadB];
+#pragma unroll
+                for (int g = 0; g < kAheadB; ++g) {
+                    q[g] = min(e + g * stride, hi - 1);
+                    s[g] = make_float3(E[q[g]], E[capk + q[g]], E[2 * capk + q[g]]);
                 }
+#pragma unroll
+                for (int g = 0; g < kAheadB; ++g) h[g] = batch_gather(a, Tp, s[g]);
+#pragma unroll
+                for (int g = 0; g < kAheadB; ++g)
+                    n[g] = make_float3(E[3 * capk + q[g]], E[4 * capk + q[g]], E[5 * capk + q[g]]);
+#pragma unroll
+                for (int g = 0; g < kAheadB; ++g)
+                    if (e + g * stride < hi) batch_accumulate(a, Tp, gate2, s[g], n[g], h[g], accr, inl);
             }
             float v[32];
 #pragma unroll
@@ -361,7 +380,7 @@ __global__ void __launch_bounds__(512, 1) icp_batched_kernel(BatchArgs a) {
             const float sum = warp_reduce_scatter(v);
             if (lane < 29) {
                 if (split == 1) acc[p * kRecWords + lane] = sum;
-                else wpart[item][lane] = sum;  // items < nw here
+                else wpart[p * split + part][lane] = sum;  // items <= nw here
             }
         }
         __syncthreads();

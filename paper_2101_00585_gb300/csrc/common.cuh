@@ -71,22 +71,22 @@ __device__ __forceinline__ bool bin_point(float x, float y, float z, const upsla
     return true;
 }
 
-// The rule as a call, for the few points bin_pixel leaves to it: (row << 32) | col, or -1 outside the panorama.
+// The rule as a call, for the few points that bin_pixel leaves to it: row * cols + col, or -1 outside the panorama.
 // Out of line: the kernels bin at many places, and the rule's divisions and roots at each of them made the ICP
 // kernel's instructions a fifth longer.
-static __device__ __noinline__ long long bin_rule_cell(float x, float y, float z, upslam_pano pp) {
+static __device__ __noinline__ int bin_rule_cell(float x, float y, float z, upslam_pano pp) {
     int row, col;
     float r;
-    return bin_point(x, y, z, pp, row, col, r) ? ((long long)row << 32) | (unsigned)col : -1ll;
+    return bin_point(x, y, z, pp, row, col, r) ? row * pp.cols + col : -1;
 }
 
 // A panorama's binning rule with what the fast form below needs, made on the host (make_bin_rule).
 struct BinRule {
     upslam_pano pp;
     float r2_min, r2_max;  // sqrt_rn(r2) lies in [r_min, r_max] exactly when r2 lies in [r2_min, r2_max]
-    float az0, el0;        // pi s_az - 1/2 and el_top s_el - 1/2, in pixels
-    float az_half, az_pi;  // pi/2 s_az and pi s_az
-    float lim;             // 1/2 minus the guard; negative: the fast form is off
+    float el0;             // el_top s_el - 1/2, in pixels
+    float az[5];           // k pi/2 s_az - 1/2, k = 0..4
+    float lim_r, lim_c;    // 1/2 minus the guard, row and column; negative: the fast form is off
 };
 
 __device__ __forceinline__ float rcp_approx(float x) {  // relative error below 2^-23
@@ -100,56 +100,73 @@ __device__ __forceinline__ float rsqrt_approx(float x) {  // relative error belo
     return r;
 }
 
+// Two FP32 values operated on by one instruction, each rounded as the scalar operation rounds it.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 twice(float v) { return pack2(v, v); }
+
 // The polynomial of atan2p, fused: P(s) with atan(t) = t P(t^2), |t| <= 1.
-__device__ __forceinline__ float atan_poly(float s) {
-    float p = fmaf(0.0028662257f, s, -0.0161657367f);
-    p = fmaf(p, s, 0.0429096138f);
-    p = fmaf(p, s, -0.0752896400f);
-    p = fmaf(p, s, 0.1065626393f);
-    p = fmaf(p, s, -0.1420889944f);
-    p = fmaf(p, s, 0.1999355085f);
-    p = fmaf(p, s, -0.3333314528f);
-    return fmaf(p, s, 1.0f);
+__device__ __forceinline__ f32x2 atan_poly2(f32x2 s) {
+    f32x2 p = fma2(twice(0.0028662257f), s, twice(-0.0161657367f));
+    p = fma2(p, s, twice(0.0429096138f));
+    p = fma2(p, s, twice(-0.0752896400f));
+    p = fma2(p, s, twice(0.1065626393f));
+    p = fma2(p, s, twice(-0.1420889944f));
+    p = fma2(p, s, twice(0.1999355085f));
+    p = fma2(p, s, twice(-0.3333314528f));
+    return fma2(p, s, twice(1.0f));
 }
 
-// The pixel of an FP32 point, the same as bin_point's bit for bit, usually without its roundings: the two
-// angles are formed with approximate reciprocals and fused multiply-adds, in pixels, and the point's cell is
-// the rule's whenever both coordinates keep `guard` away from a cell's edge, `guard` being more than the two
-// forms can differ by (make_bin_rule derives it; about 4e-4 of a pixel at 1024 columns, so one point in a
-// thousand or so is binned again by the rule itself).  The range test needs no root: it compares the rounded
-// squared range with the squares' exact limits.  A point more than 45 degrees up or down, and whatever makes a
-// NaN here (a point on the axis), goes to the rule.  The rule spends two divisions, two square roots and
-// thirty-two unfused polynomial operations, about 200 instructions; this form about 55.  It bounds
-// the kernels that bin many samples a thread (the registration's steps, the batched form, the grid search).  A
-// kernel that bins once or twice a thread (projection, averaging, hole fill, consistency) keeps the rule: it
-// waits for its slowest warp, and some warp always has a point near an edge and would do both (a keyframe update
-// measured 11.0 against 10.0 us, a consistency check 22.7 against 20.7).
-__device__ __forceinline__ bool bin_pixel(float x, float y, float z, const BinRule &b, int &row, int &col) {
+// The pixel of an FP32 point, the same as bin_point's bit for bit, usually without its roundings: the two angles
+// are formed with approximate reciprocals and fused multiply-adds, in pixels, and the point's cell is the rule's
+// whenever both coordinates keep a guard away from a cell's edge, the guard being more than the two forms can
+// differ by (make_bin_rule derives it; about 3e-4 of a pixel at 1024 columns, so fewer than one point in a
+// thousand is binned again by the rule itself).  The range test needs no root: it compares the rounded squared
+// range with the squares' exact limits.  A point more than 45 degrees up or down, and whatever makes a NaN here (a
+// point on the axis), goes to the rule.  The rule spends two divisions, two square roots and thirty-two unfused
+// polynomial operations, about 200 instructions a point; this form about 70, both polynomials in one packed
+// evaluation.  It serves the kernels that bin many samples a thread (the registration's steps, the batched form,
+// the grid search).  A kernel that bins once or twice a thread (projection, averaging, hole fill, consistency)
+// keeps the rule: it waits for its slowest warp, and some warp always has a point near an edge and would do both
+// (a keyframe update measured 11.0 against 10.0 us, a consistency check 22.7 against 20.7).  Two points to an
+// instruction throughout (packed transforms and angles) was no faster in any of the three: 89.5 against 85.0 us in
+// the grid search, and the assembler contracts packed products and sums, which the rule forbids.
+//
+// Returns row * cols + col, or -1 outside the panorama.
+__device__ __forceinline__ int bin_pixel(float x, float y, float z, const BinRule &b) {
     const float xy2 = __fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y));
     const float z2 = __fmul_rn(z, z);
     const float r2 = __fadd_rn(xy2, z2);
-    if (!(r2 >= b.r2_min && r2 <= b.r2_max)) return false;
+    if (!(r2 >= b.r2_min && r2 <= b.r2_max)) return -1;
     const float te = z * rsqrt_approx(xy2);
-    const float fr = fmaf(-(te * b.pp.s_el), atan_poly(te * te), b.el0);
-    const bool swap = fabsf(y) > fabsf(x);
+    const bool swap = fabsf(y) > fabsf(x), back = y < 0.0f;
     const float ta = (swap ? -x : y) * rcp_approx(swap ? y : x);
-    const float k = swap ? b.az_half : (x < 0.0f ? b.az_pi : 0.0f);
-    const float fc = fmaf(-(ta * b.pp.s_az), atan_poly(ta * ta), b.az0 - copysignf(k, y));
-    // nearest integer of f - 1/2 (the cell) and the distance from the cell's middle, both exact
+    const float b_swap = back ? b.az[3] : b.az[1], b_neg = back ? b.az[4] : b.az[0];
+    float pr, pc;
+    unpack2(atan_poly2(pack2(te * te, ta * ta)), pr, pc);
+    const float fr = fmaf(te * -b.pp.s_el, pr, b.el0);
+    const float fc = fmaf(ta * -b.pp.s_az, pc, swap ? b_swap : (x < 0.0f ? b_neg : b.az[2]));
     constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
     const float mr = __fadd_rn(fr, kMagic), mc = __fadd_rn(fc, kMagic);
     const float dr = __fsub_rn(fr, __fsub_rn(mr, kMagic)), dc = __fsub_rn(fc, __fsub_rn(mc, kMagic));
-    row = __float_as_int(mr) - __float_as_int(kMagic);
-    col = __float_as_int(mc) - __float_as_int(kMagic);
-    const bool in_rows = (unsigned)row < (unsigned)b.pp.rows;
-    // (NaN distances fail these tests, so they go to the rule)
-    const bool sure = z2 <= xy2 && fabsf(dr) <= b.lim &&
-                      (!in_rows || (fabsf(dc) <= b.lim && (unsigned)col < (unsigned)b.pp.cols));
-    if (__builtin_expect(sure, 1)) return in_rows;
-    const long long cell = bin_rule_cell(x, y, z, b.pp);
-    row = (int)(cell >> 32);
-    col = (int)cell;
-    return cell >= 0;
+    const int row = __float_as_int(mr) - __float_as_int(kMagic), col = __float_as_int(mc) - __float_as_int(kMagic);
+    const bool in = (unsigned)row < (unsigned)b.pp.rows;
+    const bool sure = z2 <= xy2 && fabsf(dr) <= b.lim_r &&
+                      (!in || (fabsf(dc) <= b.lim_c && (unsigned)col < (unsigned)b.pp.cols));
+    if (__builtin_expect(sure, 1)) return in ? row * b.pp.cols + col : -1;
+    return bin_rule_cell(x, y, z, b.pp);
 }
 
 // Pose rounded to FP32, row-major [R | t].
@@ -789,26 +806,23 @@ __device__ __forceinline__ bool warp_se3_update(double x, double *T, float *Tf, 
 // formed this way is exact and does not depend on the order of the additions (integer atomics from any number
 // of CTAs give every reader the same bits).
 
-// X = v * 2^48 as four signed 24-bit chunks: X = c[0] + c[1] 2^24 + c[2] 2^48 + c[3] 2^72.
+// X = v * 2^48 as four 24-bit chunks (the upper one of a pair signed): X = c[0] + c[1] 2^24 + c[2] 2^48 + c[3] 2^72.
 __device__ __forceinline__ void fx_chunks24(float v, int c[4]) {
     const unsigned b = __float_as_uint(v);
-    int e = (int)((b >> 23) & 0xffu);
-    unsigned m = e == 0xff ? 0u : b & 0x7fffffu;  // (an infinity or NaN counts as the largest value)
-    if (e) m |= 0x800000u;
-    else e = 1;
-    int sh = min(e - 150 + 48, 71);  // X = m * 2^sh, |X| < 2^95
-    if (sh < 0) {
-        m = sh > -24 ? m >> -sh : 0u;
-        sh = 0;
-    }
+    const int e = (int)((b >> 23) & 0xffu);
+    // (an infinity or NaN counts as the largest value)
+    int m = (int)((e == 0xff ? 0u : b & 0x7fffffu) | (e ? 0x800000u : 0u));
+    int sh = min((e ? e : 1) - 150 + 48, 71);  // X = m * 2^sh, |X| < 2^95
+    m >>= min(max(-sh, 0), 24);
+    sh = max(sh, 0);
+    m = (int)b < 0 ? -m : m;
     const int q = sh >= 48 ? 2 : (sh >= 24 ? 1 : 0);
-    const unsigned long long y = (unsigned long long)m << (sh - 24 * q);
-    const int lo = (int)((unsigned)y & 0xffffffu), hi = (int)(y >> 24);
-    const int sl = (b >> 31) ? -lo : lo, sg = (b >> 31) ? -hi : hi;
-    c[0] = q == 0 ? sl : 0;
-    c[1] = q == 1 ? sl : (q == 0 ? sg : 0);
-    c[2] = q == 2 ? sl : (q == 1 ? sg : 0);
-    c[3] = q == 2 ? sg : 0;
+    const int r = sh - 24 * q;
+    const int lo = (int)(((unsigned)m << r) & 0xffffffu), hi = m >> (24 - r);  // m 2^r = hi 2^24 + lo
+    c[0] = q == 0 ? lo : 0;
+    c[1] = q == 1 ? lo : (q == 0 ? hi : 0);
+    c[2] = q == 2 ? lo : (q == 1 ? hi : 0);
+    c[3] = q == 2 ? hi : 0;
 }
 
 // The sum of up to 16 numbers' 24-bit chunks as three words s0 + s1 2^32 + s2 2^64, each below 2^36 in magnitude.
@@ -1091,19 +1105,20 @@ static inline bool upslam_pano_ok(const upslam_pano *pp) {
 
 // The binning rule of a panorama for bin_pixel.
 //
-// Guard: the largest amount by which the rule's column or row coordinate and bin_pixel's can differ.  With
-// u = 2^-24 (one rounding), on the ratio t = min / max of an octant (|t| <= 1, |d atan / dt| t <= 1/2):
-//   atan, the rule: t one division (3e-8; for the row also a root, 6e-8), the unfused polynomial (1.92 u of its
-//     partial sums: 1.2e-7), its product with t and the square's rounding (6e-8): 2.4e-7 rad;
-//   atan, bin_pixel: t from an approximate reciprocal or reciprocal root (1e-7), the fused polynomial (8e-8),
-//     its products (1.1e-7): 2.9e-7 rad;
-//   column: the rule rounds pi/2 - a, pi - a and pi - az (4.2e-7 rad) and the product with s_az (u fc);
-//     bin_pixel rounds az0, az_half or az_pi, their difference and the sum (4 u of at most 2 pi s_az each);
-//   row: the rule rounds el_top - el and the product with s_el; bin_pixel rounds el0 and the sum: 4 u of at
-//     most (|el_top| + pi/2) s_el.
-// Together below 2.9e-6 rad s_az and (5.3e-7 + 2.4e-7 (|el_top| + 1.6)) rad s_el; both are taken with a fifth
-// more.  A panorama whose coordinates reach 2^20 pixels or whose guard passes a quarter of a pixel, and an
-// unlimited range, take the rule for every point.
+// Guard: the largest amount by which the rule's column or row coordinate and bin_pixel's can differ, in radians,
+// with u = 2^-24 (one rounding, relative to the value; a ratio t in [0, 1] enters atan by at most half its relative
+// error):
+//   atan, the rule: the division u/2 (for a row also the root: u), the square 0.15 u, the unfused polynomial's
+//     partial sums 1.92 u, its product with t u/2: 3.1 u (row 3.6 u);
+//   atan, bin_pixel: the approximate reciprocal (2^-23, or 2^-22.9 for a reciprocal root) and its product 1.7 u, the
+//     square 0.15 u, the fused polynomial 1.35 u, the product with t s 0.8 u: 4.0 u;
+//   column: the rule rounds pi/2 - a (u), pi - a (2 u), pi - az (4 u) and the product with s_az (2 pi u);
+//     bin_pixel rounds az[k] and the sum (2 pi u each): 25.9 u;
+//   row: the rule rounds el_top - el and the product with s_el, bin_pixel el0 and the sum: 4 u of at most
+//     |el_top| + pi/4.
+// Together below 33 u = 2.0e-6 for a column and (7.6 + 4 (|el_top| + 0.79)) u for a row; a tenth more is taken.
+// A panorama whose coordinates reach 2^20 pixels or whose guard passes a quarter of a pixel, and an unlimited
+// range, take the rule for every point.
 static inline upslam::BinRule make_bin_rule(const upslam_pano &pp) {
     upslam::BinRule b;
     b.pp = pp;
@@ -1125,16 +1140,15 @@ static inline upslam::BinRule make_bin_rule(const upslam_pano &pp) {
     b.r2_min = lo;
     b.r2_max = hi;
     const double s_az = pp.s_az, s_el = pp.s_el, top = pp.el_top;
-    b.az0 = (float)((double)upslam::kPiF * s_az - 0.5);
     b.el0 = (float)(top * s_el - 0.5);
-    b.az_half = (float)((double)upslam::kHalfPiF * s_az);
-    b.az_pi = (float)((double)upslam::kPiF * s_az);
-    const double g_az = 3.5e-6 * s_az, g_el = (6.4e-7 + 2.9e-7 * (fabs(top) + 1.6)) * s_el;
-    const double g = (g_az > g_el ? g_az : g_el) + 1e-6;
+    for (int k = 0; k < 5; ++k) b.az[k] = (float)(k * (double)upslam::kHalfPiF * s_az - 0.5);
+    const double u = 1.0 / 16777216.0;
+    const double g_c = 1.1 * 33.0 * u * s_az, g_r = 1.1 * (7.6 + 4.0 * (fabs(top) + 0.79)) * u * s_el;
     const double most = 1048576.0;
     const bool on = pp.rows < most && pp.cols < most && 6.4 * s_az < most && (fabs(top) + 1.6) * s_el < most &&
-                    g < 0.25 && hi <= FLT_MAX;
-    b.lim = on ? (float)(0.5 - g) : -1.0f;
+                    g_c < 0.25 && g_r < 0.25 && hi <= FLT_MAX;
+    b.lim_c = on ? (float)(0.5 - g_c) : -1.0f;
+    b.lim_r = on ? (float)(0.5 - g_r) : -1.0f;
     return b;
 }
 

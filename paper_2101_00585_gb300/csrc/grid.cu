@@ -128,21 +128,18 @@ __global__ void __launch_bounds__(kGridThreads) grid_score_kernel(GridArgs g, in
             for (int e = warp; e < ns; e += kGridWarps) {
                 const float3 s = make_float3(sx[e], sy[e], sz[e]);
                 const float3 q = xform_inv(T, s.x, s.y, s.z);
-                int jv, ju;
-                if (!bin_pixel(q.x, q.y, q.z, g.srule, jv, ju)) continue;
-                const int j = jv * g.sp.cols + ju;
-                const float4 P = __ldg(g.spix + j);
-                const float4 mm = load_nw(g.snrm, j, g.sprec);
-                if (P.w == 0.0f || mm.w == 0.0f) continue;
+                const int cell = bin_pixel(q.x, q.y, q.z, g.srule);
+                if (cell < 0) continue;
+                const float4 P = __ldg(g.spix + cell);
+                const float4 mm = load_nw(g.snrm, cell, g.sprec);
                 const float *R = T.r;
                 const float px = fmaf(R[0], P.x, fmaf(R[1], P.y, fmaf(R[2], P.z, R[3])));
                 const float py = fmaf(R[4], P.x, fmaf(R[5], P.y, fmaf(R[6], P.z, R[7])));
                 const float pz = fmaf(R[8], P.x, fmaf(R[9], P.y, fmaf(R[10], P.z, R[11])));
-                const float3 Rm = rotate(T, mm.x, mm.y, mm.z);
                 const float ex = px - s.x, ey = py - s.y, ez = pz - s.z;
-                const bool ok = (ex * ex + ey * ey + ez * ez <= g.d_max2) &&
-                                (Rm.x * snx[e] + Rm.y * sny[e] + Rm.z * snz[e] >= g.cos_min);
-                cnt += ok ? 1u : 0u;
+                const float3 Rm = rotate(T, mm.x, mm.y, mm.z);
+                cnt += (P.w != 0.0f) & (mm.w != 0.0f) & (ex * ex + ey * ey + ez * ez <= g.d_max2) &
+                       (Rm.x * snx[e] + Rm.y * sny[e] + Rm.z * snz[e] >= g.cos_min);
             }
         }
     }
@@ -270,10 +267,11 @@ extern "C" upslam_status upslam_grid_score(const upslam_keyframe *kf, const upsl
     g.scores = reinterpret_cast<unsigned long long *>(d_scores);
     if (cudaMemsetAsync(d_scores, 0, (size_t)n * sizeof(uint64_t), s) != cudaSuccess) return UPSLAM_ERR_CUDA;
     const int64_t ms = (int64_t)g.rows_s * g.cols_s;
-    // enough CTA columns that the launch covers every SM about four times over, each column at least one
-    // slice; every column then stages its slices kGridChunk pixels per round
+    // as many CTA columns as give every SM at most four CTAs, each column at least one slice; every column then
+    // stages its slices kGridChunk pixels per round.  (Rounded up instead, 729 candidates made 621 CTAs for 152
+    // SMs, and the SMs with five of them set the time: 106 against 92 us.)
     const int64_t slices = (ms + kGridSlice - 1) / kGridSlice;
-    int64_t xb = (4LL * upslam_sm_count() + cand_blocks - 1) / cand_blocks;
+    int64_t xb = 4LL * upslam_sm_count() / cand_blocks;
     xb = xb < 1 ? 1 : (xb > slices ? slices : xb);
     const int64_t per_round = (int64_t)xb * (kGridChunk / kGridSlice);
     const int rounds = (int)((slices + per_round - 1) / per_round);

@@ -134,7 +134,8 @@ __device__ __forceinline__ void accumulate_pixel(const IcpArgs &a, const PoseF &
     const float3 s = pixel_point(a.kdirs, a.kp.rows, v, u, d);
     const float3 q = xform_inv(T, s.x, s.y, s.z);
     int jv, ju;
-    if (!bin_pixel(q.x, q.y, q.z, a.srule, jv, ju)) return;
+    float rr;
+    if (!bin_point(q.x, q.y, q.z, a.sp, jv, ju, rr)) return;
     const int j = jv * a.sp.cols + ju;
     const float4 P = __ldcg(a.spix + j);
     if (P.w == 0.0f) return;
@@ -357,10 +358,10 @@ struct SweepHit {
 
 __device__ __forceinline__ SweepHit gather_entry(const IcpArgs &a, const PoseF &T, float3 s) {
     const float3 q = xform_inv(T, s.x, s.y, s.z);
-    int jv = 0, ju = 0;
+    const int cell = bin_pixel(q.x, q.y, q.z, a.srule);
     SweepHit h;
-    h.binned = bin_pixel(q.x, q.y, q.z, a.srule, jv, ju);
-    const int j = h.binned ? jv * a.sp.cols + ju : 0;
+    h.binned = cell >= 0;
+    const int j = cell >= 0 ? cell : 0;
     h.P = __ldcg(a.spix + j);
     h.m = load_nw_cg(a.snrm, j, a.sprec);
     return h;
@@ -405,7 +406,7 @@ __device__ __forceinline__ void accumulate_entry(const IcpArgs &a, const PoseF &
 
 // The CTA's contribution to one step's sums, exact, in two parts around a __syncthreads.  First each warp reduces
 // its 28 FP32 sums (reduce-scatter) and its two counts and leaves them in sw[warp]; then warp w adds the 16 warps'
-// sums w and w + 16 (one warp's to a lane, as 24-bit chunks with integer reductions) and lanes 0..2 and 16..18
+// sums w and w + 16 (one warp's to a lane, as 24-bit chunks) and lanes 0..2 and 16..18
 // hold the words of those two sums.
 __device__ __forceinline__ void tile_warp_sums(float acc[28], int inl, int valid, float *sw) {
     const int lane = threadIdx.x & 31;
@@ -429,17 +430,14 @@ __device__ __forceinline__ int tile_cta_word(const float (*sw)[kSumPitch], long 
         c[0] = __float_as_int(v);
         c[1] = c[2] = c[3] = 0;
     }
-    int r[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int lo = __reduce_add_sync(0xffffffffu, lane < 16 ? c[k] : 0);
-        const int hi = __reduce_add_sync(0xffffffffu, lane < 16 ? 0 : c[k]);
-        r[k] = lane < 16 ? lo : hi;
-    }
+    for (int o = 8; o >= 1; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) c[k] += __shfl_xor_sync(0xffffffffu, c[k], o);
     long long w[3];
-    fx_words(r[0], r[1], r[2], r[3], w);
+    fx_words(c[0], c[1], c[2], c[3], w);
     const int k = lane & 15;
-    word = k == 0 ? (i >= 28 ? (long long)r[0] : w[0]) : (k == 1 ? w[1] : w[2]);
+    word = k == 0 ? (i >= 28 ? (long long)c[0] : w[0]) : (k == 1 ? w[1] : w[2]);
     if (i < 28) return k < 3 ? 3 * i + k : -1;
     return i < 30 && k == 0 ? 84 + i - 28 : -1;
 }
