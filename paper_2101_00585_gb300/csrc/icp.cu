@@ -334,7 +334,9 @@ __global__ void __launch_bounds__(kIcpThreads) icp_step_kernel(IcpArgs a, double
 // prefix, so the order and therefore the sums are deterministic).  Every
 // Gauss-Newton step then reads the staged points from shared memory and gathers
 // only the sweep pixel each one lands in.  Units beyond the shared-memory
-// capacity are read from global memory each step.
+// capacity keep their samples in tensor memory, each thread its own pixel's in
+// kTmSlots slots of eight words (256 KB an SM that nothing else here uses);
+// what passes both is read from global memory each step.
 
 constexpr int kTileThreads = 512;
 constexpr int kTileWarps = kTileThreads / 32;
@@ -364,6 +366,16 @@ __device__ __forceinline__ SweepHit gather_entry(const IcpArgs &a, const PoseF &
     const int j = cell >= 0 ? cell : 0;
     h.P = __ldcg(a.spix + j);
     h.m = load_nw_cg(a.snrm, j, a.sprec);
+    return h;
+}
+
+// The same for a sample in tensor memory (word 7: its pixel index + 1, 0 for none).
+__device__ __forceinline__ SweepHit gather_slot(const IcpArgs &a, const PoseF &T, const unsigned w[8]) {
+    SweepHit h;
+    h.binned = false;
+    h.P = h.m = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (w[7] != 0u)
+        h = gather_entry(a, T, make_float3(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2])));
     return h;
 }
 
@@ -442,6 +454,38 @@ __device__ __forceinline__ int tile_cta_word(const float (*sw)[kSumPitch], long 
     return i < 30 && k == 0 ? 84 + i - 28 : -1;
 }
 
+// Tensor memory as a store of samples.  A warp reaches the 32 lanes of its quarter (its rank mod 4); of the 512
+// columns the four warps of a quarter take 128 each, so a thread owns 128 words: kTmSlots slots of eight.
+constexpr int kTmSlots = 16;
+constexpr int kTmCols = 512;
+
+__device__ __forceinline__ void tm_alloc(unsigned *base) {  // one warp
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(base)),
+                 "r"(kTmCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tm_free(unsigned base) {  // the same warp
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(kTmCols) : "memory");
+}
+__device__ __forceinline__ unsigned tm_slot(unsigned base, int slot) {
+    const int warp = threadIdx.x >> 5;
+    return base + ((unsigned)((warp & 3) * 32) << 16) + (unsigned)((warp >> 2) * (kTmCols / 4) + slot * 8);
+}
+__device__ __forceinline__ void tm_store(unsigned addr, const unsigned v[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr), "r"(v[0]),
+                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+__device__ __forceinline__ void tm_load(unsigned addr, unsigned v[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(addr)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 // Grid barrier on a monotonic 64-bit arrival counter, called by one thread per
 // CTA after a __syncthreads.  The release add publishes everything the CTA
 // wrote before the barrier; the polls are relaxed loads, and one acquire fence
@@ -497,8 +541,10 @@ __device__ __forceinline__ bool cta_grid_await(IcpCtrl *ctrl, unsigned long long
 // every CTA sums all records and solves redundantly: identical arithmetic on
 // identical data gives every CTA the same pose, so no CTA waits for another
 // to broadcast it.  CTA 0 writes the pose and the record at the end.  L1: the IRLS
-// reading of Eq. 1; KF16: the keyframe stores FP16 normals and counts.
-template <int L1, int KF16>
+// reading of Eq. 1; KF16: the keyframe stores FP16 normals and counts; SPILL: the keyframe's pixels per CTA may
+// exceed its shared memory (without it, the ordinary sizes are spared the code that follows up what did not fit:
+// 96.3 against 99.3 us for a 16x512 sweep, 100.1 against 102.2 for 64x1024).
+template <int L1, int KF16, int SPILL>
 __global__ void __launch_bounds__(kTileThreads, 1)
     icp_tile_kernel(IcpArgs a, double *pose, upslam_icp_params ip, upslam_icp_stats *st, IcpCtrl *ctrl,
                     float *partials, int cap, PriorArgs pr, FuseView fz, int fuse_on, FrontArgs fr) {
@@ -521,15 +567,18 @@ __global__ void __launch_bounds__(kTileThreads, 1)
     };
     __shared__ double tot[32];
     __shared__ long long totn[2];
+    // a step's warp sums; before the steps, the staging's counts per group, unit and warp in the same words
     __shared__ float swarp[kTileWarps][kSumPitch];
+    int (*const wcnt)[kStageGroup][kTileWarps] = reinterpret_cast<int (*)[kStageGroup][kTileWarps]>(&swarp[0][0]);
+    static_assert(2 * kStageGroup * kTileWarps <= kTileWarps * kSumPitch, "the staging's counts fit the warp sums");
     __shared__ int gbm_s;
     __shared__ double Tsh[12];
     __shared__ double Tprev[12], Tmot[12];
     __shared__ float Tf[12];
     __shared__ int acc_ok_s;
     __shared__ double xi_sh[6];
-    __shared__ int wcnt[2][kStageGroup][kTileWarps];
     __shared__ int flag, status_s, conv_s, valid_s;
+    __shared__ unsigned tm_base_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int npx = a.kp.rows * a.kp.cols;
     const int nslices = (npx + kSlice - 1) / kSlice;
@@ -661,7 +710,7 @@ __global__ void __launch_bounds__(kTileThreads, 1)
                 const int o = total + before;
                 total += __shfl_sync(0xffffffffu, incl, kTileWarps - 1);
                 off[g] = o + __popc(bal[g] & ((1u << lane) - 1u));
-                if (fit == kStageGroup && total > cap) fit = g;
+                if (SPILL && fit == kStageGroup && total > cap) fit = g;
                 if (fit == kStageGroup) staged = total;
             }
 #pragma unroll
@@ -697,6 +746,79 @@ __global__ void __launch_bounds__(kTileThreads, 1)
         }
     };
 
+    // The units that no longer fit go to tensor memory: a slot per unit in which the warp's pixels hold a sample
+    // (units of empty rows take none), as the sample's point, normal (three floats, or the keyframe's halves) and
+    // pixel index + 1 (0: this lane's pixel holds none).  tm_next is the warp's first unit left to global memory.
+    int tm_n = 0, tm_next = my_units;
+    bool tm_on = false;  // the same in every thread: the CTA holds tensor memory
+    auto tm_stage = [&]() {
+        tm_next = spill_u;
+        if (!SPILL || !spilled) return;
+        tm_on = true;
+        __syncwarp();
+        if (warp == 0) tm_alloc(&tm_base_s);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        constexpr int kB = 4;  // units loaded together
+        while (tm_next < my_units && tm_n < kTmSlots) {
+            float d[kB];
+            float4 n4[kB];
+            uint2 hv[kB];
+#pragma unroll
+            for (int g = 0; g < kB; ++g) {
+                int k;
+                const bool in = tm_next + g < my_units && unit_pixel(tm_next + g, k);
+                d[g] = in ? __ldg(a.kdepth + k) : 0.0f;
+            }
+#pragma unroll
+            for (int g = 0; g < kB; ++g) {
+                int k;
+                unit_pixel(tm_next + g, k);
+                n4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+                hv[g] = make_uint2(0u, 0u);
+                if (d[g] > 0.0f) {
+                    n4[g] = load_nw(a.knw, k, kf16 ? UPSLAM_F16 : UPSLAM_F32);
+                    if (kf16) hv[g] = __ldg(reinterpret_cast<const uint2 *>(a.knw) + k);
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < kB; ++g) {
+                if (tm_next >= my_units || tm_n >= kTmSlots) break;  // (the same in every lane)
+                const bool ok = d[g] > 0.0f && __fadd_rn(__fadd_rn(__fmul_rn(n4[g].x, n4[g].x), __fmul_rn(n4[g].y, n4[g].y)),
+                                                          __fmul_rn(n4[g].z, n4[g].z)) > 0.25f;
+                if (__any_sync(0xffffffffu, ok)) {
+                    unsigned w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+                    if (ok) {
+                        int k;
+                        unit_pixel(tm_next, k);
+                        const int v = k / W;
+                        const float3 s = pixel_point(a.kdirs, a.kp.rows, v, k - v * W, d[g]);
+                        w[0] = __float_as_uint(s.x);
+                        w[1] = __float_as_uint(s.y);
+                        w[2] = __float_as_uint(s.z);
+                        w[3] = kf16 ? hv[g].x : __float_as_uint(n4[g].x);
+                        w[4] = kf16 ? hv[g].y : __float_as_uint(n4[g].y);
+                        w[5] = kf16 ? 0u : __float_as_uint(n4[g].z);
+                        w[7] = (unsigned)k + 1u;
+                    }
+                    __syncwarp();
+                    tm_store(tm_slot(tm_base_s, tm_n), w);
+                    ++tm_n;
+                }
+                ++tm_next;
+            }
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    };
+    auto tm_release = [&]() {  // reached by the whole CTA
+        if (!SPILL || !tm_on) return;
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (warp == 0) tm_free(tm_base_s);
+    };
+
     // ---- sweep front end (upslam_track_scan): project; arrive; stage the first half of
     // the keyframe while the other CTAs finish projecting; wait; resolve the z-buffer and
     // form the normals from it in one pass; arrive; stage the rest; wait; reset the words.
@@ -714,8 +836,12 @@ __global__ void __launch_bounds__(kTileThreads, 1)
     // (one loop, so that the staging's code exists once: without a front end its single pass stages everything)
     for (int half = fr.on ? 0 : 1; half < 2; ++half) {
         stage_groups(half == 0 || !fr.on ? 0 : my_groups / 2, half == 0 ? my_groups / 2 : my_groups);
+        if (half == 1) tm_stage();
         if (!fr.on) break;
-        if (!cta_grid_await(ctrl, base + G * ++nbar, st, &flag, a.wait_cycles)) return;
+        if (!cta_grid_await(ctrl, base + G * ++nbar, st, &flag, a.wait_cycles)) {
+            tm_release();
+            return;
+        }
         const int ns = a.sp.rows * a.sp.cols;
         const int stride = gridDim.x * kTileThreads;
         if (half == 0) {
@@ -763,7 +889,33 @@ __global__ void __launch_bounds__(kTileThreads, 1)
                 h = h1;
             }
         }
-        for (int u = spill_u; u < my_units; ++u) {
+        // the samples in tensor memory, pipelined the same way (every lane of a warp goes through all slots)
+        if (SPILL && tm_n > 0) {
+            __syncwarp();
+            unsigned w[8];
+            tm_load(tm_slot(tm_base_s, 0), w);
+            SweepHit h = gather_slot(as, T, w);
+            for (int t = 0; t < tm_n; ++t) {
+                unsigned w1[8];
+                SweepHit h1 = h;
+                __syncwarp();
+                tm_load(tm_slot(tm_base_s, min(t + 1, tm_n - 1)), w1);
+                if (t + 1 < tm_n) h1 = gather_slot(as, T, w1);
+                float3 n;
+                if (kf16) {
+                    const float2 lo = __half22float2(*reinterpret_cast<const __half2 *>(&w[3]));
+                    n = make_float3(lo.x, lo.y, __low2float(*reinterpret_cast<const __half2 *>(&w[4])));
+                } else {
+                    n = make_float3(__uint_as_float(w[3]), __uint_as_float(w[4]), __uint_as_float(w[5]));
+                }
+                accumulate_entry<L1>(as, T, make_float3(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2])),
+                                     n, h, acc, inl);
+                h = h1;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) w[q] = w1[q];
+            }
+        }
+        for (int u = SPILL ? tm_next : my_units; u < my_units; ++u) {
             int k;
             if (unit_pixel(u, k)) accumulate_pixel<L1>(as, T, k, acc, inl);
         }
@@ -858,12 +1010,16 @@ __global__ void __launch_bounds__(kTileThreads, 1)
             }
         }
         __syncthreads();
-        if (flag == 3) return;
+        if (flag == 3) {
+            tm_release();
+            return;
+        }
         if (status_s != UPSLAM_OK || conv_s) {
             ++it;
             break;
         }
     }
+    tm_release();
     // the motion update M = T_prev^-1 T, by warp 0 of CTA 0
     auto publish_motion = [&]() {
         if (blockIdx.x == 0 && warp == 0 && pr.mode != 0 && pr.motion_out) {
@@ -901,14 +1057,30 @@ __global__ void __launch_bounds__(kTileThreads, 1)
             const int es = blockIdx.x == 0 ? kTileThreads - ex : kTileThreads;
             for (int e = e0; e >= 0 && e < staged; e += es)
                 fuse_average(fz, T, sk[e], make_float3(sx[e], sy[e], sz[e]), staged_nw(e), fz.kdepth[sk[e]]);
-            for (int u = spill_u; u < my_units; ++u) {
-                int k;
-                if (!unit_pixel(u, k)) continue;
-                const float4 n4 = load_nw(fz.knw, k, fz.kprec);
-                if (!(n4.w > 0.0f)) continue;
-                const float d = __ldg(fz.kdepth + k);
-                const int v = k / W;
-                fuse_average(fz, T, k, pixel_point(fz.kdirs, fz.kp.rows, v, k - v * W, d), n4, d);
+            constexpr int kB = 4;  // units loaded together
+            for (int u0 = SPILL ? spill_u : my_units; u0 < my_units; u0 += kB) {
+                float d[kB];
+                float4 n4[kB];
+#pragma unroll
+                for (int g = 0; g < kB; ++g) {
+                    int k;
+                    const bool in = u0 + g < my_units && unit_pixel(u0 + g, k);
+                    d[g] = in ? __ldcg(fz.kdepth + k) : 0.0f;
+                }
+#pragma unroll
+                for (int g = 0; g < kB; ++g) {
+                    int k;
+                    unit_pixel(u0 + g, k);
+                    n4[g] = d[g] > 0.0f ? load_nw(fz.knw, k, fz.kprec) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int g = 0; g < kB; ++g) {
+                    if (!(n4[g].w > 0.0f)) continue;
+                    int k;
+                    unit_pixel(u0 + g, k);
+                    const int v = k / W;
+                    fuse_average(fz, T, k, pixel_point(fz.kdirs, fz.kp.rows, v, k - v * W, d[g]), n4[g], d[g]);
+                }
             }
             // hole fill, first pass: z-buffer atomics into empty keyframe pixels
             for (int j = (int)(blockIdx.x * kTileThreads + threadIdx.x) - ex; j >= 0 && j < ns;
@@ -1018,31 +1190,14 @@ static upslam_status launch_tile(const IcpArgs &a, double *pose, const upslam_ic
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (!coop) return UPSLAM_ERR_UNSUPPORTED;
-    // per device and kernel variant: the kernel's static shared memory, recorded when its dynamic
-    // limit is raised (once, so later calls under stream capture change no attribute); any host
-    // thread may call, so the flags are atomic (the release store publishes static_smem)
-    static std::atomic<bool> attr_set[4][64];
-    static size_t static_smem[4][64] = {{0}};
+    // per device and kernel variant: whether the kernel's dynamic limit has been raised (once, so later
+    // calls under stream capture change no attribute); any host thread may call, so the flags are atomic
+    static std::atomic<bool> attr_set[8][64];
     if (dev < 0 || dev >= 64) return UPSLAM_ERR_UNSUPPORTED;
-    const int var = (a.l1 ? 1 : 0) + (a.kprec == UPSLAM_F16 ? 2 : 0);
-    const void *const kernels[4] = {(const void *)icp_tile_kernel<0, 0>, (const void *)icp_tile_kernel<1, 0>,
-                                    (const void *)icp_tile_kernel<0, 1>, (const void *)icp_tile_kernel<1, 1>};
-    const void *fn = kernels[var];
-    const size_t reserve = 1024;
-    if (!attr_set[var][dev].load(std::memory_order_acquire)) {
-        static std::mutex mu;
-        std::lock_guard<std::mutex> lock(mu);
-        if (!attr_set[var][dev].load(std::memory_order_relaxed)) {
-            cudaFuncAttributes fa;
-            if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) return UPSLAM_ERR_CUDA;
-            const int dyn_max = optin - (int)fa.sharedSizeBytes - (int)reserve;
-            if (dyn_max <= 0 ||
-                cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_max) != cudaSuccess)
-                return UPSLAM_ERR_UNSUPPORTED;
-            static_smem[var][dev] = fa.sharedSizeBytes;
-            attr_set[var][dev].store(true, std::memory_order_release);
-        }
-    }
+    // shared memory kept from the staged samples (the kernel's own variables and slack).  A fixed figure: what is
+    // staged decides which thread adds a sample and so the order of the sums, and stays the same whatever the
+    // kernel's variables come to.
+    constexpr int kReserve = 3296;
     const int grid = upslam_sm_count();
     if (grid > kFxMaxCtas) return UPSLAM_ERR_UNSUPPORTED;
     const int64_t npx = (int64_t)a.kp.rows * a.kp.cols;
@@ -1050,11 +1205,28 @@ static upslam_status launch_tile(const IcpArgs &a, double *pose, const upslam_ic
     const int64_t per = (nslices + grid - 1) / grid * kSlice;  // most pixels one CTA can stage
     // each staged sample: point (3), normal and count (4 floats, or 4 halves for an FP16 keyframe), pixel index
     const int64_t kWords = a.kprec == UPSLAM_F16 ? 6 : 8;
-    const int64_t cap_max =
-        (((int64_t)optin - (int64_t)static_smem[var][dev] - (int64_t)reserve) / (kWords * (int64_t)sizeof(float))) &
-        ~(int64_t)3;
+    const int64_t cap_max = (((int64_t)optin - kReserve) / (kWords * (int64_t)sizeof(float))) & ~(int64_t)3;
     const int64_t per4 = (per + 3) & ~(int64_t)3;
     const int cap = (int)(per4 < cap_max ? (per4 > 0 ? per4 : 4) : cap_max);
+    const int var = (a.l1 ? 1 : 0) + (a.kprec == UPSLAM_F16 ? 2 : 0) + (per > cap ? 4 : 0);
+    const void *const kernels[8] = {(const void *)icp_tile_kernel<0, 0, 0>, (const void *)icp_tile_kernel<1, 0, 0>,
+                                    (const void *)icp_tile_kernel<0, 1, 0>, (const void *)icp_tile_kernel<1, 1, 0>,
+                                    (const void *)icp_tile_kernel<0, 0, 1>, (const void *)icp_tile_kernel<1, 0, 1>,
+                                    (const void *)icp_tile_kernel<0, 1, 1>, (const void *)icp_tile_kernel<1, 1, 1>};
+    const void *fn = kernels[var];
+    if (!attr_set[var][dev].load(std::memory_order_acquire)) {
+        static std::mutex mu;
+        std::lock_guard<std::mutex> lock(mu);
+        if (!attr_set[var][dev].load(std::memory_order_relaxed)) {
+            cudaFuncAttributes fa;
+            if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) return UPSLAM_ERR_CUDA;
+            const int dyn_max = optin - kReserve;
+            if (dyn_max <= 0 || (int)fa.sharedSizeBytes > kReserve ||
+                cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_max) != cudaSuccess)
+                return UPSLAM_ERR_UNSUPPORTED;
+            attr_set[var][dev].store(true, std::memory_order_release);
+        }
+    }
     const size_t dyn = (size_t)cap * kWords * sizeof(float);
     if (kCtrlBytes + 2 * (size_t)grid * kSlots * sizeof(float) > ws_bytes) return UPSLAM_ERR_CAPACITY;
     int per_sm = 0;
