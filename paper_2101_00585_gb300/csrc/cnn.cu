@@ -201,6 +201,35 @@ __device__ __forceinline__ TcUnit tc_unit(const TcGemm &g, int u) {
     return t;
 }
 
+// Boxes of the A operand that hold nothing the product needs are not loaded (the TMA engine's requests, one per box
+// row, pace these GEMMs): in the forward of the first layer the 16 features of a tap row above the window (ty = 0,
+// dy = 0: a zero weight whatever the input), whose MMA is skipped too, and past the last feature; in a weight
+// gradient the same features and the rows past the feature of ones, whose products the epilogue drops.
+template <int LA>
+__device__ __forceinline__ bool tc_box_unused(const TcOperand &a, int f) {
+    if (LA == LD_S2D_KT) return (f >> 4) == 0 || (f >> 4) == 2;
+    if (LA == LD_S2D_MNT) return (f >> 4) == 2;  // (box 0 is the feature of ones)
+    if (LA == LD_IM2COL_KT32) return f >= a.kf;
+    if (LA == LD_IM2COL_MNT || LA == LD_IM2COL_MNT32) return f >= a.kf && f != a.ones_row;
+    return false;
+}
+
+// Bytes of one K step's boxes (those of B whole; of A without the boxes left out).
+template <int LA, int BN>
+__device__ __forceinline__ unsigned tc_step_bytes(const TcOperand &a, const TcUnit &t, int k0) {
+    constexpr bool KM = LA == LD_S2D_KT || LA == LD_IM2COL_KT32;  // boxes along K
+    constexpr int CB = LA == LD_S2D_KT || LA == LD_S2D_MNT ? 16 : tma_cb<LA>();
+    constexpr int kAll = KM ? kTcBK / CB : kTcBM / CB;
+    constexpr unsigned kBox = (unsigned)((kTcBM * kTcBK * 2) / kAll);
+    unsigned bytes = (unsigned)((kTcBM + BN) * kTcBK * 2);
+    if (KM || LA == LD_S2D_MNT || LA == LD_IM2COL_MNT || LA == LD_IM2COL_MNT32) {
+#pragma unroll
+        for (int h = 0; h < kAll; ++h)
+            if (tc_box_unused<LA>(a, (KM ? k0 : t.r0a) + CB * h)) bytes -= kBox;
+    }
+    return bytes;
+}
+
 // TMA loads of the A operand of one K step (tensor maps built on the host; coordinates past the tensor read as
 // zeros).  The data gradient's:
 //   A, LD_DY_TAPS_K: class pixels (b, i, j) from t.r0a by (tap, n) from k0: one box [128 rows][128 B] in the
@@ -225,6 +254,7 @@ __device__ __forceinline__ void tc_tma_a(unsigned stage, unsigned mbar, const Tc
 #pragma unroll 1
         for (int h = 0; h < (FWD ? 4 : 8); ++h) {
             const int f = (FWD ? k0 : t.r0a) + 16 * h;
+            if (tc_box_unused<LA>(a, f)) continue;
             const unsigned dst = stage + h * (FWD ? 4096 : 2048);
             if (!FWD && f == a.ones_row) {
                 tma_load4(dst, mo, 0, 0, 0, 0, mbar);
@@ -244,6 +274,7 @@ __device__ __forceinline__ void tc_tma_a(unsigned stage, unsigned mbar, const Tc
 #pragma unroll 1
         for (int h = 0; h < kTcBM / CB; ++h) {
             const int f = t.r0a + CB * h;
+            if (tc_box_unused<LA>(a, f)) continue;
             if (f == a.ones_row) {
                 tma_load4(stage + h * CB * 128, mo, 0, 0, 0, 0, mbar);
                 continue;
@@ -270,6 +301,7 @@ __device__ __forceinline__ void tc_tma_a(unsigned stage, unsigned mbar, const Tc
 #pragma unroll 1
         for (int h = 0; h < kTcBK / CB; ++h) {
             const int f = k0 + CB * h;
+            if (tc_box_unused<LA>(a, f)) continue;
             int c0 = 0, c1 = 0, c2 = 0, c3 = a.nb;
             if (f < a.kf) {
                 const int tap = f >> a.cs, ky = tap / 3, kx = tap - 3 * ky;
@@ -481,7 +513,6 @@ __global__ void __launch_bounds__(kTcThreads, 2)
     constexpr int S = tc_stages<BN>();
     static_assert(S >= 2 && S <= 8, "stage ring");
     constexpr int kA = kTcBM * kTcBK * 2, kStage = (kTcBM + BN) * kTcBK * 2;
-    constexpr unsigned kTxBytes = (unsigned)kStage;  // TMA boxes are written in full (zeros outside)
     constexpr bool A_MN = LA == LD_IM2COL_MNT || LA == LD_IM2COL_MNT32 || LA == LD_S2D_MNT;
     constexpr bool B_MN = LB == LD_W_TAPS_MN || LB == LD_DENSE_MNT || LB == LD_DENSE_MNT32;
     extern __shared__ __align__(1024) unsigned char tc_smem[];
@@ -512,6 +543,10 @@ __global__ void __launch_bounds__(kTcThreads, 2)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = sy.tmem_base;
+    // the set-up above overlapped the kernel before (programmatic dependent launch); its results are read from here
+    // on, and the next kernel may set up in turn
+    pdl_wait();
+    pdl_release();
 
     if (warp == 4) {
         // ---- producer (one thread)
@@ -529,7 +564,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
                     }
                     const unsigned stage = smem0 + st * kStage, fb = smem_u32(&sy.full[st]);
                     const int k0 = t.kbeg + k * kTcBK;
-                    mbar_expect_tx(fb, kTxBytes);
+                    mbar_expect_tx(fb, tc_step_bytes<LA, BN>(g.a, t, k0));
                     tc_tma_a<LA>(stage, fb, g.a, &tma_a, &tma_one, t, k0);
                     tc_tma_b<LB, BN>(stage + kA, fb, g.b, &tma_b, t, k0);
                 }
@@ -580,6 +615,9 @@ __global__ void __launch_bounds__(kTcThreads, 2)
                     const int k0 = t.kbeg + k * kTcBK;
                     const int nk = min(kTcBK / 16, (t.kend - k0 + 15) / 16);
                     for (int kk = 0; kk < nk; ++kk) {
+                        // (its 16 features were not loaded; the first features of all are left out, so the first
+                        // MMA of a unit is the one that does not accumulate)
+                        if (LA == LD_S2D_KT && tc_box_unused<LA>(g.a, k0 + 16 * kk)) continue;
                         // TMA tiles: A K-major 128-byte swizzle (an MMA's 16 k start 32 bytes along the row); B
                         // MN-major, 128-byte swizzle (BN >= 64: 8-row K groups 1024 B apart, 64-channel atoms
                         // 8 KB apart) or 64-byte swizzle (BN = 32: K groups 512 B apart); an MMA spans two K groups
@@ -600,7 +638,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
                             : LB == LD_DENSE_MNT32 ? umma_desc_sw(b0 + kk * 1024, 512, 512, 4)
                             : BN == 32           ? umma_desc_sw(b0 + kk * 1024, 512, 512, 4)
                                                  : umma_desc_sw(b0 + kk * 2048, 8192, 1024, 2);
-                        const unsigned accum = (k > 0 || kk > 0) ? 1u : 0u;
+                        const unsigned accum = (k > 0 || kk > (LA == LD_S2D_KT ? 1 : 0)) ? 1u : 0u;
                         asm volatile(
                             "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
                             " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc),
@@ -661,13 +699,23 @@ __global__ void __launch_bounds__(kTcThreads, 2)
 
 // Global mean over [B, HW, C = 128] (BF16) -> g [B, C] (FP32), then the linear head out = g W^T + b.
 // 128 threads per sample: thread t sums channels 8 (t % 16) .. + 7 over pixels t / 16, t / 16 + 8, ... with
-// 16-byte loads; the eight partial sums of each channel are folded in shared memory.
+// 16-byte loads; the eight partial sums of each channel are folded in shared memory.  The head's weights are
+// staged in shared memory while the pixels arrive: six threads then walk the 128 channels in order (read from
+// global memory one by one they took most of the kernel's 9.9 us for one sample).
 __global__ void __launch_bounds__(128) pool_head_kernel(const __nv_bfloat16 *__restrict__ x, int B, int HW, int C,
                                                         const float *wf, const float *bf, float *g, float *out) {
     const int b = blockIdx.x, t = threadIdx.x, c8 = (t & 15) * 8, p0 = t >> 4;
     __shared__ float part[8][128];
     __shared__ float gs[128];
+    __shared__ float ws[6][129];
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float wt[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) wt[i] = __ldg(wf + i * C + t);
+    const float bias = t < 6 ? __ldg(bf + t) : 0.0f;
+    pdl_wait();  // the last layer's output is complete
+    pdl_release();
+#pragma unroll 8
     for (int p = p0; p < HW; p += 8) {
         const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x + ((long long)b * HW + p) * C + c8));
         const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
@@ -680,6 +728,8 @@ __global__ void __launch_bounds__(128) pool_head_kernel(const __nv_bfloat16 *__r
     }
 #pragma unroll
     for (int q = 0; q < 8; ++q) part[p0][c8 + q] = acc[q];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) ws[i][t] = wt[i];
     __syncthreads();
     float sum = 0.0f;
 #pragma unroll
@@ -688,8 +738,9 @@ __global__ void __launch_bounds__(128) pool_head_kernel(const __nv_bfloat16 *__r
     g[b * C + t] = sum / HW;
     __syncthreads();
     if (t < 6) {
-        float o = bf[t];
-        for (int c = 0; c < C; ++c) o += wf[t * C + c] * gs[c];
+        float o = bias;
+#pragma unroll 16
+        for (int c = 0; c < 128; ++c) o += ws[t][c] * gs[c];
         out[b * 6 + t] = o;
     }
 }
@@ -707,6 +758,7 @@ __global__ void __launch_bounds__(128) head_backward_kernel(const float *out, co
     __shared__ float dout[kHeadB][6];
     __shared__ float lsum;
     const int t = threadIdx.x;
+    pdl_release();  // (the next kernel waits for this one before it reads anything)
     if (t == 0) lsum = 0.0f;
     __syncthreads();
     if (t < kHeadB * 6) {
@@ -746,6 +798,8 @@ __global__ void __launch_bounds__(128) head_backward_kernel(const float *out, co
 __global__ void __launch_bounds__(256) head_dy_kernel(const float *__restrict__ dg, const __nv_bfloat16 *__restrict__ x4,
                                                       int B, int HW, __nv_bfloat16 *__restrict__ dy4) {
     const int total = B * HW * 16;
+    pdl_wait();  // the pooled features' gradient is complete
+    pdl_release();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const int c = (i & 15) << 3, pix = i >> 4, b = pix / HW;
         const uint4 xm = __ldg(reinterpret_cast<const uint4 *>(x4) + i);
@@ -774,6 +828,7 @@ struct PackArgs {
     int n[4];
 };
 __global__ void pack_weights_kernel(PackArgs a) {
+    pdl_release();  // the first layer may set up meanwhile
     const int total = a.n[0] + a.n[1] + a.n[2] + a.n[3];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         int l = 0, k = i;
@@ -1088,8 +1143,8 @@ static bool gemm(TcGemm g, int *err, cudaStream_t s, int splits = 1) {
             return false;
     }
     const int cap = 2 * upslam_sm_count();  // persistent: two CTAs per SM
-    gemm_tc_kernel<EPI, BN, LA, LB><<<g.units < cap ? g.units : cap, kTcThreads, smem, s>>>(g, err, ma, mb, mo);
-    return true;
+    return launch_dependent(gemm_tc_kernel<EPI, BN, LA, LB>, dim3(g.units < cap ? g.units : cap), dim3(kTcThreads),
+                            smem, s, g, err, ma, mb, mo);
 }
 
 }  // namespace upslam
@@ -1174,9 +1229,10 @@ static upslam_status cnn_forward(const float *d_params, const void *d_x, int32_t
         H /= 2;
         W /= 2;
     }
-    pool_head_kernel<<<batch, 128, 0, s>>>(w.act[3], batch, H * W, 128, d_params + L.off_wf, d_params + L.off_bf, w.g,
-                                           d_out);
     UPSLAM_CHECK_LAUNCH();
+    if (!launch_dependent(pool_head_kernel, dim3(batch), dim3(128), 0, s, (const __nv_bfloat16 *)w.act[3], batch, H * W,
+                          128, d_params + L.off_wf, d_params + L.off_bf, w.g, d_out))
+        return UPSLAM_ERR_CUDA;
     return UPSLAM_OK;
 }
 
@@ -1211,7 +1267,10 @@ extern "C" upslam_status upslam_cnn_backward(const float *d_params, const void *
                                                                        d_params + L.off_wf, 4 * 16,
                                                                        d_grads + L.off_wf, d_grads + L.off_bf, w.dg,
                                                                        d_loss);
-    head_dy_kernel<<<grid1d((long long)batch * 64 * 16), 256, 0, s>>>(w.dg, w.act[3], batch, 4 * 16, w.dy[3]);
+    UPSLAM_CHECK_LAUNCH();
+    if (!launch_dependent(head_dy_kernel, dim3(grid1d((long long)batch * 64 * 16)), dim3(256), 0, s, (const float *)w.dg,
+                          (const __nv_bfloat16 *)w.act[3], batch, 4 * 16, w.dy[3]))
+        return UPSLAM_ERR_CUDA;
     const int sms = upslam_sm_count();
     for (int l = 3; l >= 0; --l) {
         const int C = kCnnCh[l], N = cnn_co(l), K = cnn_k(l);

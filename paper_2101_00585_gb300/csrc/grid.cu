@@ -202,17 +202,19 @@ __global__ void __launch_bounds__(1024) grid_best_kernel(const unsigned long lon
 }
 
 // poses[i] = exp(xi_i^) * center (left update, FP64), xi_i = (omega, v) in FP32.
-__global__ void grid_candidates_kernel(const double *center, const float *xi, int n, double *poses) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per candidate: a dozen dependent FP64 instructions, where one thread's took about ninety at 64 cycles each.
+__global__ void __launch_bounds__(128) grid_candidates_kernel(const double *center, const float *xi, int n,
+                                                              double *poses) {
+    __shared__ double Ts[4][12];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x * 4 + warp;
     if (i >= n) return;
-    double T[12], x[6];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) T[k] = __ldg(center + k);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) x[k] = (double)__ldg(xi + (size_t)i * 6 + k);
-    se3_exp_left(x, T);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) poses[(size_t)i * 12 + k] = T[k];
+    double *T = Ts[warp];
+    if (lane < 12) T[lane] = __ldg(center + lane);
+    const double x = f2d(lane < 6 ? __ldg(xi + (size_t)i * 6 + lane) : 0.0f);
+    __syncwarp();
+    (void)warp_se3_update(x, T, nullptr, 0.0, 0.0);
+    if (lane < 12) poses[(size_t)i * 12 + lane] = T[lane];
 }
 
 }  // namespace upslam
@@ -223,7 +225,7 @@ extern "C" upslam_status upslam_grid_candidates(const double *d_center12, const 
                                                 double *d_poses, void *stream) {
     if (!d_center12 || !d_xi || !d_poses || n < 0) return UPSLAM_ERR_INVALID_ARG;
     if (n == 0) return UPSLAM_OK;
-    grid_candidates_kernel<<<(n + 127) / 128, 128, 0, (cudaStream_t)stream>>>(d_center12, d_xi, n, d_poses);
+    grid_candidates_kernel<<<(n + 3) / 4, 128, 0, (cudaStream_t)stream>>>(d_center12, d_xi, n, d_poses);
     UPSLAM_CHECK_LAUNCH();
     return UPSLAM_OK;
 }

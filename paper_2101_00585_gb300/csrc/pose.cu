@@ -71,13 +71,19 @@ extern "C" upslam_status upslam_update_motion(const double *d_T_prev, const doub
 
 namespace upslam {
 
-__global__ void se3_exp_batch_kernel(const float *xi, int n, double *poses) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per twist (warp_se3_update: a dozen dependent FP64 instructions, where one thread's took about ninety at
+// 64 cycles each).
+__global__ void __launch_bounds__(128) se3_exp_batch_kernel(const float *xi, int n, double *poses) {
+    __shared__ double Ts[4][12];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x * 4 + warp;
     if (i >= n) return;
-    double x[6], T[12] = {1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0};
-    for (int k = 0; k < 6; ++k) x[k] = (double)xi[6 * i + k];
-    se3_exp_left(x, T);
-    for (int k = 0; k < 12; ++k) poses[12 * i + k] = T[k];
+    double *T = Ts[warp];
+    if (lane < 12) T[lane] = lane % 5 == 0 ? 1.0 : 0.0;
+    const double x = f2d(lane < 6 ? __ldg(xi + 6 * (size_t)i + lane) : 0.0f);
+    __syncwarp();
+    (void)warp_se3_update(x, T, nullptr, 0.0, 0.0);
+    if (lane < 12) poses[12 * (size_t)i + lane] = T[lane];
 }
 
 }  // namespace upslam
@@ -85,7 +91,7 @@ __global__ void se3_exp_batch_kernel(const float *xi, int n, double *poses) {
 extern "C" upslam_status upslam_se3_exp(const float *d_xi, int32_t n, double *d_poses, void *stream) {
     if (!d_xi || !d_poses || n < 0) return UPSLAM_ERR_INVALID_ARG;
     if (n == 0) return UPSLAM_OK;
-    se3_exp_batch_kernel<<<(n + 127) / 128, 128, 0, (cudaStream_t)stream>>>(d_xi, n, d_poses);
+    se3_exp_batch_kernel<<<(n + 3) / 4, 128, 0, (cudaStream_t)stream>>>(d_xi, n, d_poses);
     UPSLAM_CHECK_LAUNCH();
     return UPSLAM_OK;
 }
