@@ -16,12 +16,19 @@ from . import _abi
 F32, F16 = _abi.F32, _abi.F16
 
 
+# the current stream's handle without the Stream object around it, where torch offers it (one call instead of four
+# Python frames; every entry point asks once per call)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _p(t: torch.Tensor | None):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _require_cuda(*ts):
@@ -454,15 +461,16 @@ def keyframe_consistency(kf_a: "KeyframeBuffer", kf_b: "KeyframeBuffer", T_ab: t
     L = _abi.lib()
     ka, kb = kf_a.struct(), kf_b.struct()
     nbytes = int(L.upslam_consistency_workspace_bytes(ctypes.byref(ka), ctypes.byref(kb)))
-    ws = torch.zeros(nbytes, dtype=torch.uint8, device=T_ab.device)
-    removed = torch.zeros(2, dtype=torch.int64, device=T_ab.device)
+    # (every flag and both counts are written by the call: nothing to clear)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=T_ab.device)
+    removed = torch.empty(2, dtype=torch.int64, device=T_ab.device)
     _abi.check("upslam_keyframe_consistency",
                L.upslam_keyframe_consistency(ctypes.byref(ka), ctypes.byref(kb), _p(T_ab.contiguous()), float(rel),
                                              float(abs_m), _p(ws), nbytes, _p(removed), _stream()))
     Ha, Wa = int(kf_a.pp.rows), int(kf_a.pp.cols)
     Hb, Wb = int(kf_b.pp.rows), int(kf_b.pp.cols)
     off_b = (Ha * Wa + 255) // 256 * 256
-    return removed, ws[:Ha * Wa].view(Ha, Wa), ws[off_b:off_b + Hb * Wb].view(Hb, Wb)
+    return removed, ws.as_strided((Ha, Wa), (Wa, 1)), ws.as_strided((Hb, Wb), (Wb, 1), off_b)
 
 
 # ----------------------------------------------------------------------------- batched registration
