@@ -946,6 +946,16 @@ __global__ void __launch_bounds__(kTileThreads, 1)
             unsigned long long w[3];
             const long long t0 = clock64();
             bool late = false;
+            // first one word, the CTA's own choice of the 86, until its count is full: 152 CTAs reading all words all
+            // the while delay the adds they wait for (94.7 against 86.4 us for a 16x512 sweep of 11 steps)
+            for (;;) {
+                asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];"
+                             : "=l"(w[0])
+                             : "l"(buf + (size_t)(blockIdx.x % kFxWords) * kAccStride)
+                             : "memory");
+                if ((w[0] >> 48) == G || clock64() - t0 > a.wait_cycles) break;
+            }
+            __syncwarp();
             for (;;) {
                 bool done = true;
 #pragma unroll
