@@ -144,12 +144,13 @@ __device__ __forceinline__ f32x2 atan_poly2(f32x2 s) {
 // instruction throughout (packed transforms and angles) was no faster in any of the three: 89.5 against 85.0 us in
 // the grid search, and the assembler contracts packed products and sums, which the rule forbids.
 //
-// Returns row * cols + col, or -1 outside the panorama.
-__device__ __forceinline__ int bin_pixel(float x, float y, float z, const BinRule &b) {
+// bin_fast: cell = row * cols + col, or -1 outside the panorama; false when the rule has to decide.  No branch, so that
+// a caller's other work fills its dependent chain.
+__device__ __forceinline__ bool bin_fast(float x, float y, float z, const BinRule &b, int &cell) {
     const float xy2 = __fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y));
     const float z2 = __fmul_rn(z, z);
     const float r2 = __fadd_rn(xy2, z2);
-    if (!(r2 >= b.r2_min && r2 <= b.r2_max)) return -1;
+    const bool in_range = (r2 >= b.r2_min) & (r2 <= b.r2_max);
     const float te = z * rsqrt_approx(xy2);
     const bool swap = fabsf(y) > fabsf(x), back = y < 0.0f;
     const float ta = (swap ? -x : y) * rcp_approx(swap ? y : x);
@@ -162,11 +163,19 @@ __device__ __forceinline__ int bin_pixel(float x, float y, float z, const BinRul
     const float mr = __fadd_rn(fr, kMagic), mc = __fadd_rn(fc, kMagic);
     const float dr = __fsub_rn(fr, __fsub_rn(mr, kMagic)), dc = __fsub_rn(fc, __fsub_rn(mc, kMagic));
     const int row = __float_as_int(mr) - __float_as_int(kMagic), col = __float_as_int(mc) - __float_as_int(kMagic);
-    const bool in = (unsigned)row < (unsigned)b.pp.rows;
-    const bool sure = z2 <= xy2 && fabsf(dr) <= b.lim_r &&
-                      (!in || (fabsf(dc) <= b.lim_c && (unsigned)col < (unsigned)b.pp.cols));
-    if (__builtin_expect(sure, 1)) return in ? row * b.pp.cols + col : -1;
-    return bin_rule_cell(x, y, z, b.pp);
+    const bool in = in_range & ((unsigned)row < (unsigned)b.pp.rows);
+    cell = in ? row * b.pp.cols + col : -1;
+    // (NaN distances fail these tests, so they go to the rule)
+    const bool row_sure = (z2 <= xy2) & (fabsf(dr) <= b.lim_r);
+    const bool col_sure = (fabsf(dc) <= b.lim_c) & ((unsigned)col < (unsigned)b.pp.cols);
+    return !in_range | (row_sure & (!in | col_sure));
+}
+
+// The cell, with the rule where it has to decide.
+__device__ __forceinline__ int bin_pixel(float x, float y, float z, const BinRule &b) {
+    int cell;
+    if (__builtin_expect(!bin_fast(x, y, z, b, cell), 0)) cell = bin_rule_cell(x, y, z, b.pp);
+    return cell;
 }
 
 // Pose rounded to FP32, row-major [R | t].

@@ -358,15 +358,19 @@ struct SweepHit {
     bool binned;
 };
 
-__device__ __forceinline__ SweepHit gather_entry(const IcpArgs &a, const PoseF &T, float3 s) {
-    const float3 q = xform_inv(T, s.x, s.y, s.z);
-    const int cell = bin_pixel(q.x, q.y, q.z, a.srule);
+// The sweep data of the pixel `cell` (-1: none; the first pixel is read and dropped).
+__device__ __forceinline__ SweepHit gather_cell(const IcpArgs &a, int cell) {
     SweepHit h;
     h.binned = cell >= 0;
     const int j = cell >= 0 ? cell : 0;
     h.P = __ldcg(a.spix + j);
     h.m = load_nw_cg(a.snrm, j, a.sprec);
     return h;
+}
+
+__device__ __forceinline__ SweepHit gather_entry(const IcpArgs &a, const PoseF &T, float3 s) {
+    const float3 q = xform_inv(T, s.x, s.y, s.z);
+    return gather_cell(a, bin_pixel(q.x, q.y, q.z, a.srule));
 }
 
 // The same for a sample in tensor memory (word 7: its pixel index + 1, 0 for none).
