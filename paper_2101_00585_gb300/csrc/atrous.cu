@@ -98,21 +98,13 @@ extern "C" upslam_status upslam_atrous_normals(const upslam_pano *pp, const floa
     const void *src = d_nrm_in;
     for (int l = 0; l < ap->levels; ++l) {
         void *dst = ((ap->levels - 1 - l) % 2 == 0) ? d_nrm_out : d_tmp;
-        if (l == 0) {
-            if (precision == UPSLAM_F32)
-                atrous_kernel<UPSLAM_F32><<<blocks, 64, 0, s>>>(*pp, pix, src, dst, 1 << l, inv_sn2, inv_sx2);
-            else
-                atrous_kernel<UPSLAM_F16><<<blocks, 64, 0, s>>>(*pp, pix, src, dst, 1 << l, inv_sn2, inv_sx2);
-            UPSLAM_CHECK_LAUNCH();
-        } else {
-            // later levels overlap the previous level's tail (each waits for its input first)
-            const bool ok = precision == UPSLAM_F32
-                                ? launch_dependent(atrous_kernel<UPSLAM_F32>, dim3(blocks), dim3(64), 0, s, *pp, pix,
-                                                   src, dst, 1 << l, inv_sn2, inv_sx2)
-                                : launch_dependent(atrous_kernel<UPSLAM_F16>, dim3(blocks), dim3(64), 0, s, *pp, pix,
-                                                   src, dst, 1 << l, inv_sn2, inv_sx2);
-            if (!ok) return UPSLAM_ERR_CUDA;
-        }
+        // each level overlaps the tail of the launch before it (it waits for its input first)
+        const bool ok = precision == UPSLAM_F32
+                            ? launch_dependent(atrous_kernel<UPSLAM_F32>, dim3(blocks), dim3(64), 0, s, *pp, pix, src,
+                                               dst, 1 << l, inv_sn2, inv_sx2)
+                            : launch_dependent(atrous_kernel<UPSLAM_F16>, dim3(blocks), dim3(64), 0, s, *pp, pix, src,
+                                               dst, 1 << l, inv_sn2, inv_sx2);
+        if (!ok) return UPSLAM_ERR_CUDA;
         src = dst;
     }
     return UPSLAM_OK;

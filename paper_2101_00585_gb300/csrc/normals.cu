@@ -15,6 +15,8 @@ namespace upslam {
 __global__ void __launch_bounds__(256) normals_kernel(const float4 *__restrict__ pix, const float *__restrict__ depth,
                                                       upslam_pano pp, upslam_normal_params np, void *nrm,
                                                       int precision) {
+    pdl_wait();     // the pixels are resolved
+    pdl_release();  // and the smoothing may place its CTAs
     const int npx = pp.rows * pp.cols;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < npx; k += gridDim.x * blockDim.x)
         store_nw(nrm, k, precision, normal_pixel(PixArrays<false>{pix, depth}, pp, np, k));
@@ -32,8 +34,8 @@ extern "C" upslam_status upslam_normals(const float *d_pix, const float *d_depth
     if (nrm_precision != UPSLAM_F32 && nrm_precision != UPSLAM_F16) return UPSLAM_ERR_INVALID_ARG;
     if (!upslam_aligned(d_nrm, nrm_precision == UPSLAM_F32 ? 16 : 8)) return UPSLAM_ERR_INVALID_ARG;
     const int npx = pp->rows * pp->cols;
-    normals_kernel<<<upslam_grid(npx, 256), 256, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const float4 *>(d_pix), d_depth, *pp, *np, d_nrm, nrm_precision);
-    UPSLAM_CHECK_LAUNCH();
-    return UPSLAM_OK;
+    return launch_dependent(normals_kernel, dim3(upslam_grid(npx, 256)), dim3(256), 0, (cudaStream_t)stream,
+                            reinterpret_cast<const float4 *>(d_pix), d_depth, *pp, *np, d_nrm, (int)nrm_precision)
+               ? UPSLAM_OK
+               : UPSLAM_ERR_CUDA;
 }

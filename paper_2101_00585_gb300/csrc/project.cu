@@ -58,7 +58,8 @@ __global__ void __launch_bounds__(256) project_kernel(const float4 *__restrict__
 __global__ void __launch_bounds__(256) resolve_kernel(const float4 *__restrict__ pts, int npx,
                                                       unsigned long long *__restrict__ zbuf, float *__restrict__ depth,
                                                       int *__restrict__ idx, float4 *__restrict__ pix) {
-    pdl_wait();  // every point of the projection has reached the z-buffer
+    pdl_wait();     // every point of the projection has reached the z-buffer
+    pdl_release();  // and the normals may place their CTAs
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < npx; k += gridDim.x * blockDim.x)
         resolve_pixel<false>(pts, k, zbuf, depth, idx, pix);
 }
