@@ -244,7 +244,8 @@ __device__ __forceinline__ void tc_tma_a(unsigned stage, unsigned mbar, const Tc
     if (LA == LD_S2D_KT || LA == LD_S2D_MNT) {
         // boxes of 16 features (one dy of a tap: 32-byte rows, 32-byte swizzle) over the NHWC input read as
         // [B][H][W/2][16], at (X, y) = (ox + tx - 1, 2 (oy + ty - 1) + dy); padding reads zeros.  Forward:
-        // rows = 128 output pixels from t.r0a, the K step's 64 features = 4 boxes [128][32 B] 4 KB apart.
+        // rows = 128 output pixels from t.r0a, the K step's 64 features = 4 boxes [128][32 B] 4 KB apart (the two of
+        // zero weights left out: 52.4 -> 46.3 us at batch 256).
         // Weight gradient: k = 64 output pixels from k0, rows = the 128 features as 8 boxes [64][32 B] 2 KB
         // apart, the first box the feature of ones.
         constexpr bool FWD = LA == LD_S2D_KT;
@@ -267,7 +268,7 @@ __device__ __forceinline__ void tc_tma_a(unsigned stage, unsigned mbar, const Tc
     }
     if (LA == LD_IM2COL_MNT || LA == LD_IM2COL_MNT32) {
         // k: 64 pixels from k0; rows: features t.r0a.. as boxes of CB channels, [64 k][2 CB bytes] each, 128 CB
-        // bytes apart (the appended feature of ones from mo; features past it read zeros from image nb)
+        // bytes apart (the appended feature of ones from mo; features past it are not loaded)
         constexpr int CB = tma_cb<LA>();
         const int wo = a.ws - 1, ho = a.hs - 1;
         const int ox0 = k0 & ((1 << wo) - 1), oy0 = (k0 >> wo) & ((1 << ho) - 1), b0 = k0 >> (wo + ho);
@@ -294,7 +295,7 @@ __device__ __forceinline__ void tc_tma_a(unsigned stage, unsigned mbar, const Tc
     if (LA == LD_IM2COL_KT || LA == LD_IM2COL_KT32) {
         // rows: 128 output pixels from t.r0a (whole output rows); k: 64 features as boxes of CB channels of one
         // tap ([128 rows][2 CB bytes], 8 KB apart when CB = 32), each stepping 2 along W and H from
-        // (2 ox0 + kx - 1, 2 oy0 + ky - 1); the padding and features past 9 C read zeros
+        // (2 ox0 + kx - 1, 2 oy0 + ky - 1); the padding reads zeros, features past 9 C are not loaded
         constexpr int CB = tma_cb<LA>();
         const int wo = a.ws - 1, ho = a.hs - 1;
         const int ox0 = t.r0a & ((1 << wo) - 1), oy0 = (t.r0a >> wo) & ((1 << ho) - 1), b0 = t.r0a >> (wo + ho);

@@ -8,8 +8,16 @@
 // J^T J and J^T r with r = (T s2 - s1) . N(s1) and J = [p x N, N] (p = T s2,
 // left update T <- exp(xi^) T).
 //
-// The 6x6 system is solved with an FP64 square-root-free Cholesky (L D L^T)
-// and the SE(3) exponential is applied in FP64.
+// The 6x6 system is solved in FP64 (warp_solve6: by 3 x 3 blocks where they are
+// certified, else by a square-root-free Cholesky) and the SE(3) exponential is
+// applied in FP64.
+//
+// Time of one Gauss-Newton step of icp_tile_kernel (in-kernel time stamps, 64x1024
+// sweep, 190 k samples): 8.1 us (10.5 with the exact binning rule at every
+// sample, atomics for the CTA sums, a six-pivot elimination and a poll of all
+// words): accumulate 3.2 (last CTA 3.8), CTA sums 0.9, the last add to the read
+// of the totals 0.8, totals to doubles 0.3, solve 1.2, update 0.7.  What bounds it
+// is the latency of that chain; a 16x512 sweep's step takes 5.6 us (7.9).
 //
 // Two launch forms:
 //  * icp_step_kernel: one Gauss-Newton step.  FP32 per thread -> warp shuffles
@@ -19,7 +27,7 @@
 //  * icp_tile_kernel: all iterations in one cooperative launch, one CTA per SM,
 //    the CTA's keyframe samples staged in shared memory once.  Each step's sums
 //    are exact fixed-point integers that every CTA adds into global words; the
-//    same words carry an arrival count, so one poll of them is both the grid
+//    same words carry an arrival count, so reading them is both the grid
 //    barrier and the read of the totals.  Every CTA then solves the identical
 //    system itself.  Every wait is bounded by a clock64 budget and reports
 //    UPSLAM_ERR_TIMEOUT instead of hanging.
@@ -46,8 +54,8 @@ constexpr int kFxWords = 86;          // 28 sums x 3 chunks, inliers, valid
 // 64-bit words from one accumulator to the next: each sits on its own 128-byte L2 line, so the
 // adds and polls of 152 CTAs spread over many L2 slices instead of queueing on six lines
 constexpr int kAccStride = 16;
-// Each CTA adds into every accumulator of a step exactly once: its partial (a CTA's partial lies
-// in (-2^36, 2^36): 16 warps of chunks below 2^32) plus kFxBias, which makes the addend positive,
+// Each CTA adds into every accumulator of a step exactly once: its partial (a CTA's words lie
+// in (-2^36, 2^36): fx_words) plus kFxBias, which makes the addend positive,
 // plus one arrival unit in bits 48-63.  With at most kFxMaxCtas CTAs the low 48 bits never carry
 // into the count, so a word holds its whole total exactly when its count equals the grid size.
 constexpr unsigned long long kFxBias = 1ull << 36;
