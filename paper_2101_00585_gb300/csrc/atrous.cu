@@ -21,21 +21,21 @@
 namespace upslam {
 
 template <int PREC>
-__global__ void __launch_bounds__(64, 8) atrous_kernel(upslam_pano pp, const float4 *__restrict__ pix, const void *nin,
+__global__ void __launch_bounds__(64, 8) atrous_kernel(upslam_pano pp, const float4 *pix, const void *nin,
                                                       void *nout, int step, float inv_sn2, float inv_sx2) {
     pdl_wait();     // the previous level's output is complete
     pdl_release();  // and the next level may place its CTAs
     const int W = pp.cols, H = pp.rows, npx = H * W;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= npx) return;
-    const float4 n0 = load_nw(nin, k, PREC);
+    const float4 n0 = load_nw_l1(nin, k, PREC);
     if (n0.w == 0.0f) {
         store_nw(nout, k, PREC, make_float4(0.f, 0.f, 0.f, 0.f));
         return;
     }
     const float h[5] = {0.0625f, 0.25f, 0.375f, 0.25f, 0.0625f};
     const int v = k / W, u = k - v * W;
-    const float4 P = __ldg(pix + k);
+    const float4 P = pix[k];
     const float inv_scale2 = inv_sx2 / (P.x * P.x + P.y * P.y + P.z * P.z);
     float ax = 0.0f, ay = 0.0f, az = 0.0f;
     // Branch-free taps: a row outside the image reads the pixel's own row instead and an invalid tap is
@@ -50,8 +50,8 @@ __global__ void __launch_bounds__(64, 8) atrous_kernel(upslam_pano pp, const flo
             int uq = u + dx * step;
             uq = uq < 0 ? uq + W : (uq >= W ? uq - W : uq);
             const int q = vr * W + uq;
-            const float4 n = load_nw(nin, q, PREC);
-            const float4 Q = __ldg(pix + q);
+            const float4 n = load_nw_l1(nin, q, PREC);
+            const float4 Q = pix[q];
             const float ex = n0.x - n.x, ey = n0.y - n.y, ez = n0.z - n.z;
             const float dn2 = ex * ex + ey * ey + ez * ez;
             const float dpl = n0.x * (Q.x - P.x) + n0.y * (Q.y - P.y) + n0.z * (Q.z - P.z);

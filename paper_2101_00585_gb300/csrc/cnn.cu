@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(128) pool_head_kernel(const __nv_bfloat16 *__r
     pdl_release();
 #pragma unroll 8
     for (int p = p0; p < HW; p += 8) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x + ((long long)b * HW + p) * C + c8));
+        const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(x + ((long long)b * HW + p) * C + c8));
         const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -804,8 +804,8 @@ __global__ void __launch_bounds__(256) head_dy_kernel(const float *__restrict__ 
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const int c = (i & 15) << 3, pix = i >> 4, b = pix / HW;
         const uint4 xm = __ldg(reinterpret_cast<const uint4 *>(x4) + i);
-        const float4 lo = __ldg(reinterpret_cast<const float4 *>(dg + b * 128 + c));
-        const float4 hi = __ldg(reinterpret_cast<const float4 *>(dg + b * 128 + c) + 1);
+        const float4 lo = __ldcg(reinterpret_cast<const float4 *>(dg + b * 128 + c));
+        const float4 hi = __ldcg(reinterpret_cast<const float4 *>(dg + b * 128 + c) + 1);
         const float v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
         const __nv_bfloat162 *xh = reinterpret_cast<const __nv_bfloat162 *>(&xm);
         uint4 o;

@@ -250,13 +250,23 @@ __device__ __forceinline__ float3 pixel_point(const float *dirs, int rows, int v
 
 // ----------------------------------------------------------------------------- storage helpers
 
-__device__ __forceinline__ float4 load_nw(const void *base, int64_t k, int precision) {
-    if (precision == UPSLAM_F32) return __ldg(reinterpret_cast<const float4 *>(base) + k);
-    const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(base) + k);
+__device__ __forceinline__ float4 unpack_nw(uint2 raw) {
     const __half2 a = *reinterpret_cast<const __half2 *>(&raw.x);
     const __half2 b = *reinterpret_cast<const __half2 *>(&raw.y);
     const float2 fa = __half22float2(a), fb = __half22float2(b);
     return make_float4(fa.x, fa.y, fb.x, fb.y);
+}
+
+__device__ __forceinline__ float4 load_nw(const void *base, int64_t k, int precision) {
+    if (precision == UPSLAM_F32) return __ldg(reinterpret_cast<const float4 *>(base) + k);
+    return unpack_nw(__ldg(reinterpret_cast<const uint2 *>(base) + k));
+}
+
+// Same load, an ordinary one through L1 (for data that the launch before may still write when this kernel's CTAs are
+// placed).
+__device__ __forceinline__ float4 load_nw_l1(const void *base, int64_t k, int precision) {
+    if (precision == UPSLAM_F32) return reinterpret_cast<const float4 *>(base)[k];
+    return unpack_nw(reinterpret_cast<const uint2 *>(base)[k]);
 }
 
 // Same load, through L2 only (for data rewritten during the kernel's lifetime by other CTAs).
@@ -919,13 +929,13 @@ __device__ __forceinline__ void resolve_pixel(const float4 *pts, int k, unsigned
     }
 }
 
-// Pixel data for the normals, read from the resolved arrays (point with validity in .w, range).
-template <bool kCg>
+// Pixel data for the normals, read from the resolved arrays (point with validity in .w, range) by ordinary loads: the
+// launch before may still be writing them when the kernel's CTAs are placed.
 struct PixArrays {
     const float4 *pix;
     const float *depth;
-    __device__ __forceinline__ float4 point(int k) const { return ld_front<kCg>(pix + k); }
-    __device__ __forceinline__ float range(int k) const { return ld_front<kCg>(depth + k); }
+    __device__ __forceinline__ float4 point(int k) const { return pix[k]; }
+    __device__ __forceinline__ float range(int k) const { return depth[k]; }
 };
 
 // The same data decoded straight from the z-buffer words (winner index and range in the key),

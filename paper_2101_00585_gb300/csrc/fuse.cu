@@ -47,6 +47,8 @@ __device__ __forceinline__ bool accepted(const upslam_icp_stats *st, float accep
     return ok != 0;
 }
 
+// (The keyframe is read through L2: the update before this one may still be writing it when these CTAs are placed, and
+// the read-only path is only for data that no launch writes while the kernel runs.)
 __global__ void __launch_bounds__(256) fuse_main_kernel(FuseView f, const double *pose, upslam_icp_stats *st, int gk) {
     pdl_wait();     // what ran before (the update before this one, say) has finished
     pdl_release();  // the hole-fill write launch may place its CTAs while this grid drains
@@ -66,12 +68,12 @@ __global__ void __launch_bounds__(256) fuse_main_kernel(FuseView f, const double
 #pragma unroll
             for (int b = 0; b < kB; ++b) {
                 const int k = base + b * blockDim.x;
-                d[b] = k < npx ? __ldg(f.kdepth + k) : 0.0f;
+                d[b] = k < npx ? __ldcg(f.kdepth + k) : 0.0f;
             }
 #pragma unroll
             for (int b = 0; b < kB; ++b) {
                 const int k = base + b * blockDim.x;
-                n[b] = d[b] > 0.0f ? load_nw(f.knw, k, f.kprec) : make_float4(0.f, 0.f, 0.f, 0.f);
+                n[b] = d[b] > 0.0f ? load_nw_cg(f.knw, k, f.kprec) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int b = 0; b < kB; ++b) {
@@ -91,7 +93,7 @@ __global__ void __launch_bounds__(256) fuse_main_kernel(FuseView f, const double
             float r;
             float4 m;
             if (!holefill_key(f, T, j, k, key, r, m)) continue;
-            if (__ldg(f.kdepth + k) > 0.0f) continue;  // a pixel holding a sample is averaged, not filled
+            if (__ldcg(f.kdepth + k) > 0.0f) continue;  // a pixel holding a sample is averaged, not filled
             atomicMin(f.zbuf + k, key);
         }
     }

@@ -12,14 +12,13 @@
 
 namespace upslam {
 
-__global__ void __launch_bounds__(256) normals_kernel(const float4 *__restrict__ pix, const float *__restrict__ depth,
-                                                      upslam_pano pp, upslam_normal_params np, void *nrm,
-                                                      int precision) {
+__global__ void __launch_bounds__(256) normals_kernel(const float4 *pix, const float *depth, upslam_pano pp,
+                                                      upslam_normal_params np, void *nrm, int precision) {
     pdl_wait();     // the pixels are resolved
     pdl_release();  // and the smoothing may place its CTAs
     const int npx = pp.rows * pp.cols;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < npx; k += gridDim.x * blockDim.x)
-        store_nw(nrm, k, precision, normal_pixel(PixArrays<false>{pix, depth}, pp, np, k));
+        store_nw(nrm, k, precision, normal_pixel(PixArrays{pix, depth}, pp, np, k));
 }
 
 }  // namespace upslam
