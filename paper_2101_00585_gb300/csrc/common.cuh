@@ -719,8 +719,10 @@ __device__ __forceinline__ bool warp_solve6(const double *tot, double pivot_eps,
     const int em = (hm >> 20) - 1023, e0 = (h0 >> 20) - 1023, e1 = (h1 >> 20) - 1023, e2 = (h2 >> 20) - 1023,
               e3 = (h3 >> 20) - 1023, e4 = (h4 >> 20) - 1023, e5 = (h5 >> 20) - 1023;
     const int low = em - 23 + 1;
+    // (d'' is a product of twelve elements, between 2^(12 em - 288) and 2^(12 em + 12) with such pivots: em keeps it
+    // and its reciprocal normal numbers.  Below, d'' underflows to zero, whose exponent field is no exponent.)
     const bool good = (h0 | h1 | h2 | h3 | h4 | h5) >= 0 && e0 >= low && e1 - e0 > low && e2 - e1 > low &&
-                      e3 - e2 > low && e4 - e3 - e2 - 1 > low && e5 - e4 - e2 - 1 > low && em > -500 && em < 100 &&
+                      e3 - e2 > low && e4 - e3 - e2 - 1 > low && e5 - e4 - e2 - 1 > low && em > -59 && em < 83 &&
                       dbits(pivot_eps) <= dbits(2.9802322387695312e-08);  // 2^-25
     if (good && __all_sync(full, dfinite(*x))) return true;
     return warp_solve6_pivots(tot, pivot_eps, x);
