@@ -653,12 +653,20 @@ constexpr unsigned long long lane_tab6(int a, int b, int c, int d, int e, int f)
 // every line a set of sums of two to four products, one sum to a lane: 21 dependent FP64 instructions and seven
 // exchanges between lanes, where the pivoting elimination above takes 30 and nineteen.  An FP64 instruction takes
 // 64 cycles of its warp whatever its active lanes, so the number on the chain is the time: 3851 cycles
-// (1.86 us) for the elimination, 2177 (1.05 us) for this form.  Largest error against 50-digit solutions over
-// condition numbers up to 1e7: 1.2e-14 here, 1.5e-14 there.  Products of minors lose more digits than an
-// elimination does when A is close to singular, so this form is taken only where every pivot (a ratio of its minors) is certain, from the
-// exponents alone, to be above 2^-24 of the largest diagonal element; otherwise, and whenever pivot_eps asks for
-// more or a value is not finite, the elimination solves the system and decides whether it is degenerate.
+// (1.86 us) for the elimination, 2177 (1.05 us) for this form.
+//
+// Which systems it solves: a difference of products is good to 2^-53 of the products, not of itself, so this form
+// loses what d is below the product of P's diagonal and what det S is below that of S's.  Both losses are read off
+// the exponents and may come to kBlockLoss bits; neither depends on the units of A's rows.  Beyond, where a pivot is
+// not certain to be above 2^-24 of the largest diagonal element, whenever pivot_eps asks for more, and when a value
+// is not finite, the elimination solves the system and decides whether it is degenerate (then both are paid for).
+// The 3062 systems of streams, registrations and batches of hypotheses on sweeps of 16x512 to 128x2048 lose one bit
+// at most; largest relative error of xi there against 113-bit solutions 7e-15 (elimination: 1.0e-14).  Of random
+// spectra in random bases, with and without rows of unlike scale, and of corridors, round tunnels, ground planes and
+// frames far from their points, the accepted ones: 4.8e-14 (5.5e-14); at five bits or more some lose more digits
+// here than there.
 // *x: lane k < 6 holds xi[k].
+constexpr int kBlockLoss = 3;
 __device__ __forceinline__ bool warp_solve6(const double *tot, double pivot_eps, double *x) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -710,19 +718,23 @@ __device__ __forceinline__ bool warp_solve6(const double *tot, double pivot_eps,
     *x = dneg(lane < 3 ? xa : xb3);
     // every pivot certainly above 2^-24 of the largest diagonal element (in [2^em, 2^(em+1)))?  The pivots are
     // P_00, minor / P_00, d / minor, S''_00 / d, minor'' / (S''_00 d), d'' / (minor'' d)
-    int hm = __double2hiint(tot[0]);
-    hm = max(max(hm, __double2hiint(tot[6])), max(__double2hiint(tot[11]), __double2hiint(tot[15])));
-    hm = max(hm, max(__double2hiint(tot[18]), __double2hiint(tot[20])));
-    const int h0 = __double2hiint(tot[0]), h1 = __shfl_sync(full, __double2hiint(c1), 5), h2 = __double2hiint(det);
+    const int d0 = __double2hiint(tot[0]), d1 = __double2hiint(tot[6]), d2 = __double2hiint(tot[11]),
+              d3 = __double2hiint(tot[15]), d4 = __double2hiint(tot[18]), d5 = __double2hiint(tot[20]);
+    const int hm = max(max(max(d0, d1), max(d2, d3)), max(d4, d5));
+    const int h1 = __shfl_sync(full, __double2hiint(c1), 5), h2 = __double2hiint(det);
     const int h3 = __shfl_sync(full, __double2hiint(sz), 0), h4 = __shfl_sync(full, __double2hiint(c2), 5),
               h5 = __double2hiint(det2);
-    const int em = (hm >> 20) - 1023, e0 = (h0 >> 20) - 1023, e1 = (h1 >> 20) - 1023, e2 = (h2 >> 20) - 1023,
+    const int em = (hm >> 20) - 1023, e0 = (d0 >> 20) - 1023, e1 = (h1 >> 20) - 1023, e2 = (h2 >> 20) - 1023,
               e3 = (h3 >> 20) - 1023, e4 = (h4 >> 20) - 1023, e5 = (h5 >> 20) - 1023;
     const int low = em - 23 + 1;
+    // bits that d is below P_00 P_11 P_22, and d'' = d^3 det S below d^3 S_00 S_11 S_22
+    const int loss1 = (d0 >> 20) + (d1 >> 20) + (d2 >> 20) - 3 * 1023 - e2;
+    const int loss2 = (d3 >> 20) + (d4 >> 20) + (d5 >> 20) - 3 * 1023 + 3 * e2 - e5;
     // (d'' is a product of twelve elements, between 2^(12 em - 288) and 2^(12 em + 12) with such pivots: em keeps it
     // and its reciprocal normal numbers.  Below, d'' underflows to zero, whose exponent field is no exponent.)
-    const bool good = (h0 | h1 | h2 | h3 | h4 | h5) >= 0 && e0 >= low && e1 - e0 > low && e2 - e1 > low &&
-                      e3 - e2 > low && e4 - e3 - e2 - 1 > low && e5 - e4 - e2 - 1 > low && em > -59 && em < 83 &&
+    const bool good = (d0 | h1 | h2 | h3 | h4 | h5) >= 0 && e0 >= low && e1 - e0 > low && e2 - e1 > low &&
+                      e3 - e2 > low && e4 - e3 - e2 - 1 > low && e5 - e4 - e2 - 1 > low && loss1 <= kBlockLoss &&
+                      loss1 + loss2 <= kBlockLoss && em > -59 && em < 83 &&
                       dbits(pivot_eps) <= dbits(2.9802322387695312e-08);  // 2^-25
     if (good && __all_sync(full, dfinite(*x))) return true;
     return warp_solve6_pivots(tot, pivot_eps, x);
