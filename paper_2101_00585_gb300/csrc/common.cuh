@@ -71,15 +71,6 @@ __device__ __forceinline__ bool bin_point(float x, float y, float z, const upsla
     return true;
 }
 
-// The rule as a call, for the few points that bin_pixel leaves to it: row * cols + col, or -1 outside the panorama.
-// Out of line: the kernels bin at many places, and the rule's divisions and roots at each of them made the ICP
-// kernel's instructions a fifth longer.
-static __device__ __noinline__ int bin_rule_cell(float x, float y, float z, upslam_pano pp) {
-    int row, col;
-    float r;
-    return bin_point(x, y, z, pp, row, col, r) ? row * pp.cols + col : -1;
-}
-
 // A panorama's binning rule with what the fast form below needs, made on the host (make_bin_rule).
 struct BinRule {
     upslam_pano pp;
@@ -134,18 +125,18 @@ __device__ __forceinline__ f32x2 atan_poly2(f32x2 s) {
 // whenever both coordinates keep a guard away from a cell's edge, the guard being more than the two forms can
 // differ by (make_bin_rule derives it; about 3e-4 of a pixel at 1024 columns, so fewer than one point in a
 // thousand is binned again by the rule itself).  The range test needs no root: it compares the rounded squared
-// range with the squares' exact limits.  A point more than 45 degrees up or down, and whatever makes a NaN here (a
-// point on the axis), goes to the rule.  The rule spends two divisions, two square roots and thirty-two unfused
-// polynomial operations, about 200 instructions a point; this form about 70, both polynomials in one packed
-// evaluation.  It serves the kernels that bin many samples a thread (the registration's steps, the batched form,
+// range with the squares' exact limits.  A point more than 45 degrees up or down takes its row from the inverse ratio
+// in bin_rest_cell, and whatever makes a NaN here (a point on the axis) goes to the rule.  The rule spends two
+// divisions, two square roots and thirty-two unfused polynomial operations, about 200 instructions a point; this form
+// about 70, both polynomials in one packed evaluation.  It serves the kernels that bin many samples a thread (the registration's steps, the batched form,
 // the grid search).  A kernel that bins once or twice a thread (projection, averaging, hole fill, consistency)
 // keeps the rule: it waits for its slowest warp, and some warp always has a point near an edge and would do both
 // (a keyframe update measured 11.0 against 10.0 us, a consistency check 22.7 against 20.7).  Two points to an
 // instruction throughout (packed transforms and angles) was no faster in any of the three: 89.5 against 85.0 us in
 // the grid search, and the assembler contracts packed products and sums, which the rule forbids.
 //
-// bin_fast: cell = row * cols + col, or -1 outside the panorama; false when the rule has to decide.  No branch, so that
-// a caller's other work fills its dependent chain.
+// bin_fast: cell = row * cols + col, or -1 outside the panorama; false when bin_rest_cell has to decide, for a point
+// within the range limits.  No branch, so that a caller's other work fills its dependent chain.
 __device__ __forceinline__ bool bin_fast(float x, float y, float z, const BinRule &b, int &cell) {
     const float xy2 = __fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y));
     const float z2 = __fmul_rn(z, z);
@@ -171,10 +162,66 @@ __device__ __forceinline__ bool bin_fast(float x, float y, float z, const BinRul
     return !in_range | (row_sure & (!in | col_sure));
 }
 
-// The cell, with the rule where it has to decide.
+// P(s) of atan_poly2, one value.
+__device__ __forceinline__ float atan_poly(float s) {
+    float p = fmaf(0.0028662257f, s, -0.0161657367f);
+    p = fmaf(p, s, 0.0429096138f);
+    p = fmaf(p, s, -0.0752896400f);
+    p = fmaf(p, s, 0.1065626393f);
+    p = fmaf(p, s, -0.1420889944f);
+    p = fmaf(p, s, 0.1999355085f);
+    p = fmaf(p, s, -0.3333314528f);
+    return fmaf(p, s, 1.0f);
+}
+
+// The pixel a coordinate rounds to; false within `guard` of a pixel's edge.
+__device__ __forceinline__ bool sure_pixel(float f, float guard, int &i) {
+    constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
+    const float m = __fadd_rn(f, kMagic);
+    i = __float_as_int(m) - __float_as_int(kMagic);
+    return fabsf(__fsub_rn(f, __fsub_rn(m, kMagic))) <= 0.5f - guard;
+}
+
+// The guards of a steep point's row and column in radians (make_bin_rule).
+__device__ __forceinline__ float bin_steep_row_guard(float el_top) {
+    return 1.1f / 16777216.0f * (10.7f + 5.0f * (fabsf(el_top) + 1.58f));
+}
+constexpr float kSteepColGuard = 1.1f * 37.0f / 16777216.0f;
+
+// What bin_fast leaves: the cell of a point steeper than 45 degrees, el = +-pi/2 - atan(rho / z), with guards of its own,
+// and the rule for the rest; row * cols + col, or -1 outside the panorama.  Out of line: the kernels bin at many
+// places, and the rule's divisions and roots at each of them made the ICP kernel's instructions a fifth longer.
+// With the rule alone here, a panorama that looks up (89 to 46 degrees, every sample steep) paid for both: 305 us for
+// 729 candidates of the grid search, where the rule at every point takes 289; now 257 (a batch 6.77 ms, 6.91, 5.81).
+// The ordinary points' time hangs on the registers that this call takes from its callers: handed bin_fast's column
+// instead of forming it again, 122.0 against 119.8 us for 14 steps on a 64x1024 sweep; with both polynomials in one
+// packed evaluation, 1 us more for 8 steps into a 1024x4096 keyframe; in this form within 0.2 us of the rule alone.
+static __device__ __noinline__ int bin_rest_cell(float x, float y, float z, upslam_pano pp) {
+    const float xy2 = __fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y));
+    int row, col;
+    if (__fmul_rn(z, z) > xy2) {
+        // (a guard of half a pixel or more, as for coordinates too large for the magic sums, leaves no point here)
+        const float te = xy2 * rsqrt_approx(xy2) * rcp_approx(z);
+        const float fr = fmaf(te * pp.s_el, atan_poly(te * te),
+                              fmaf(z > 0.0f ? -kHalfPiF : kHalfPiF, pp.s_el, fmaf(pp.el_top, pp.s_el, -0.5f)));
+        if (sure_pixel(fr, bin_steep_row_guard(pp.el_top) * pp.s_el, row)) {
+            if ((unsigned)row >= (unsigned)pp.rows) return -1;
+            const bool swap = fabsf(y) > fabsf(x);
+            const float ta = (swap ? -x : y) * rcp_approx(swap ? y : x);
+            const float quarters = swap ? (y < 0.0f ? 3.0f : 1.0f) : (x < 0.0f ? (y < 0.0f ? 4.0f : 0.0f) : 2.0f);
+            const float fc = fmaf(ta * -pp.s_az, atan_poly(ta * ta), fmaf(quarters * kHalfPiF, pp.s_az, -0.5f));
+            if (sure_pixel(fc, kSteepColGuard * pp.s_az, col) && (unsigned)col < (unsigned)pp.cols)
+                return row * pp.cols + col;
+        }
+    }
+    float r;
+    return bin_point(x, y, z, pp, row, col, r) ? row * pp.cols + col : -1;
+}
+
+// The cell.
 __device__ __forceinline__ int bin_pixel(float x, float y, float z, const BinRule &b) {
     int cell;
-    if (__builtin_expect(!bin_fast(x, y, z, b, cell), 0)) cell = bin_rule_cell(x, y, z, b.pp);
+    if (__builtin_expect(!bin_fast(x, y, z, b, cell), 0)) cell = bin_rest_cell(x, y, z, b.pp);
     return cell;
 }
 
@@ -1149,8 +1196,14 @@ static inline bool upslam_pano_ok(const upslam_pano *pp) {
 //   column: the rule rounds pi/2 - a (u), pi - a (2 u), pi - az (4 u) and the product with s_az (2 pi u);
 //     bin_pixel rounds az[k] and the sum (2 pi u each): 25.9 u;
 //   row: the rule rounds el_top - el and the product with s_el, bin_pixel el0 and the sum: 4 u of at most
-//     |el_top| + pi/4.
-// Together below 33 u = 2.0e-6 for a column and (7.6 + 4 (|el_top| + 0.79)) u for a row; a tenth more is taken.
+//     |el_top| + pi/4;
+//   row of a steep point: the rule rounds pi/2 - atan too (u); the ratio rho / z is a reciprocal root, a reciprocal
+//     and two products (6.2 u, half of it in the angle: with the rest as above 5.4 u); the base with pi/2 is one
+//     rounding more, 5 u of at most |el_top| + pi/2; and where the rule takes the other ratio (the two tests of 45
+//     degrees may differ by a rounding) the polynomial's own error counts twice, 0.7 u;
+//   column of a steep point: 3 pi/2 rounded (4 u) more than a column's.
+// Together below 33 u = 2.0e-6 for a column, (7.6 + 4 (|el_top| + 0.79)) u for a row, and 37 u and (10.7 + 5 (|el_top| +
+// 1.58)) u for a steep point's; a tenth more is taken.
 // A panorama whose coordinates reach 2^20 pixels or whose guard passes a quarter of a pixel, and an unlimited
 // range, take the rule for every point.
 static inline upslam::BinRule make_bin_rule(const upslam_pano &pp) {
