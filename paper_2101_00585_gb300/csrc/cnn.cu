@@ -702,7 +702,9 @@ __global__ void __launch_bounds__(kTcThreads, 2)
 // 128 threads per sample: thread t sums channels 8 (t % 16) .. + 7 over pixels t / 16, t / 16 + 8, ... with
 // 16-byte loads; the eight partial sums of each channel are folded in shared memory.  The head's weights are
 // staged in shared memory while the pixels arrive: six threads then walk the 128 channels in order (read from
-// global memory one by one they took most of the kernel's 9.9 us for one sample).
+// global memory one by one they took most of the kernel's 9.9 us for one sample).  Weights and bias are read before
+// the wait: whatever wrote the parameters had finished when the pass's first launch, pack_weights_kernel, began,
+// because that one is an ordinary launch.  Were it made a dependent one, these reads would have to follow the wait.
 __global__ void __launch_bounds__(128) pool_head_kernel(const __nv_bfloat16 *__restrict__ x, int B, int HW, int C,
                                                         const float *wf, const float *bf, float *g, float *out) {
     const int b = blockIdx.x, t = threadIdx.x, c8 = (t & 15) * 8, p0 = t >> 4;

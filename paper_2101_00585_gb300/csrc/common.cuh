@@ -949,13 +949,7 @@ __device__ __forceinline__ double fx_value(long long s0, long long s1, long long
 //
 // The per-point and per-pixel bodies of projection, resolve and normals, shared by
 // the standalone kernels and the fused register launch so both give the same bits.
-// kCg selects L2-only loads for data that the same launch wrote earlier (the
-// read-only cache path is only for data no launch writes while it runs).
-
-template <bool kCg, typename T>
-__device__ __forceinline__ T ld_front(const T *p) {
-    return kCg ? __ldcg(p) : __ldg(p);
-}
+// kCg selects L2-only loads for z-buffer words that the same launch wrote earlier.
 
 // Pass 1 of the z-buffer: the point's key (bits(range) << 32 | index) into its pixel.
 __device__ __forceinline__ void project_point(const float4 *pts, int i, const upslam_pano &pp,
@@ -1139,9 +1133,11 @@ __device__ __forceinline__ void holefill_write(const FuseView &f, const PoseF &T
 //
 // Where one entry point runs several kernels in a row, the later ones are launched with
 // launch_dependent: their CTAs may be placed while the kernel before them drains, and each runs
-// pdl_wait() before it reads anything (the wait returns once the previous grid has finished and its
-// writes are visible).  A kernel lets its successor start early with pdl_release(); without it the
-// successor starts at its end, as an ordinary launch would.
+// pdl_wait() before it reads anything that this kernel or one before it writes (the wait returns once the
+// previous grid has finished and its writes are visible).  A kernel lets its successor start early with
+// pdl_release(); without it the successor starts at its end, as an ordinary launch would.  A dependent
+// kernel waits before it ends, and releases after its wait; one that releases without a wait is launched
+// as an ordinary one.  So the previous grid's end is also the end of all before it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

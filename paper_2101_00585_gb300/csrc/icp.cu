@@ -1218,7 +1218,9 @@ static upslam_status launch_tile(const IcpArgs &a, double *pose, const upslam_ic
     if (dev < 0 || dev >= 64) return UPSLAM_ERR_UNSUPPORTED;
     // shared memory kept from the staged samples (the kernel's own variables and slack).  A fixed figure: what is
     // staged decides which thread adds a sample and so the order of the sums, and stays the same whatever the
-    // kernel's variables come to.
+    // kernel's variables come to.  They come to 2816 bytes; past 3296 every call below is refused as unsupported, so
+    // what would add more than the 480 bytes left has to raise the figure (and with it the order of the sums of
+    // keyframes that do not fit).
     constexpr int kReserve = 3296;
     const int grid = upslam_sm_count();
     if (grid > kFxMaxCtas) return UPSLAM_ERR_UNSUPPORTED;
