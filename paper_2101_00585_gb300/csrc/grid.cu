@@ -271,7 +271,10 @@ extern "C" upslam_status upslam_grid_score(const upslam_keyframe *kf, const upsl
     const int64_t ms = (int64_t)g.rows_s * g.cols_s;
     // as many CTA columns as give every SM at most four CTAs, each column at least one slice; every column then
     // stages its slices kGridChunk pixels per round.  (Rounded up instead, 729 candidates made 621 CTAs for 152
-    // SMs, and the SMs with five of them set the time: 106 against 92 us.)
+    // SMs, and the SMs with five of them set the time: 106 against 92 us.  Counted by the busiest SM's share, rounding
+    // down is the better or equal up to 152 blocks of candidates, rounding up between 153 and 190, 229 and 253, 305
+    // and 380; calls there, e.g. 600 us for 4913 candidates and 1409 for 9800, where the exact rule with rounding up
+    // took 781 and 1536.)
     const int64_t slices = (ms + kGridSlice - 1) / kGridSlice;
     int64_t xb = 4LL * upslam_sm_count() / cand_blocks;
     xb = xb < 1 ? 1 : (xb > slices ? slices : xb);
